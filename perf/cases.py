@@ -120,6 +120,14 @@ def _ball(gen, n, r_in, r_out):
     return d * (r_in ** 3 + u * (r_out ** 3 - r_in ** 3)) ** (1.0 / 3.0)
 
 
+def _rotations(q):
+    """Rotation matrices [N, 3, 3] of unit quaternions (r, i, j, k)."""
+    r, i, j, k = q.unbind(1)
+    return torch.stack([1 - 2 * (j * j + k * k), 2 * (i * j - r * k), 2 * (i * k + r * j),
+                        2 * (i * j + r * k), 1 - 2 * (i * i + k * k), 2 * (j * k - r * i),
+                        2 * (i * k - r * j), 2 * (j * k + r * i), 1 - 2 * (i * i + j * j)], 1).view(-1, 3, 3)
+
+
 def _scene(case, seed, n=None, isotropic=False):
     """Activated parameters as a dict of float32 CUDA tensors."""
     n = case["n"] if n is None else n
@@ -131,7 +139,7 @@ def _scene(case, seed, n=None, isotropic=False):
         means, log_s = rand(n, 3) * 2 - 1, 0.5 * randn(n, 3) - 3.0
     elif case["scene"] == "cluster":
         centres, stds = 6.0 * rand(64, 3) - 3.0, 0.05 + 0.45 * rand(64, 3)
-        frames = torch.linalg.qr(randn(64, 3, 3))[0]
+        frames = _rotations(torch.nn.functional.normalize(randn(64, 4), dim=1))
         which = torch.randint(0, 64, (n,), generator=gen, device="cuda")
         means = centres[which] + torch.einsum("nij,nj->ni", frames[which], stds[which] * randn(n, 3))
         log_s = randn(n, 3) - 4.0
@@ -422,11 +430,7 @@ def _exact_frame(p, case, cam, dimg):
     if iso:
         M = leaves["scales"][:, None, None] * torch.eye(3, dtype=torch.float64, device="cuda")
     else:
-        r, i, j, k = torch.nn.functional.normalize(leaves["quats"], dim=1).unbind(1)
-        Rq = torch.stack([1 - 2 * (j * j + k * k), 2 * (i * j - r * k), 2 * (i * k + r * j),
-                          2 * (i * j + r * k), 1 - 2 * (i * i + k * k), 2 * (j * k - r * i),
-                          2 * (i * k - r * j), 2 * (j * k + r * i), 1 - 2 * (i * i + j * j)], 1).view(-1, 3, 3)
-        M = Rq * leaves["scales"][:, None, :]
+        M = _rotations(torch.nn.functional.normalize(leaves["quats"], dim=1)) * leaves["scales"][:, None, :]
     V = J @ R @ M
     S = V @ V.transpose(1, 2) + float(np.float32(0.3)) * torch.eye(2, dtype=torch.float64, device="cuda")
     A, B, C = S[:, 0, 0], S[:, 0, 1], S[:, 1, 1]
@@ -509,10 +513,7 @@ def _exact_refine(s):
     normals = torch.randn((n, 2, 3), dtype=torch.float32, device="cuda", generator=s.gen.manual_seed(s.seed)).double()
     out = {k: t.double()[src] for k, t in p.items()}
     sp = split[src]
-    r, i, j, k = torch.nn.functional.normalize(out["quats"], dim=1).unbind(1)
-    R = torch.stack([1 - 2 * (j * j + k * k), 2 * (i * j - r * k), 2 * (i * k + r * j),
-                     2 * (i * j + r * k), 1 - 2 * (i * i + k * k), 2 * (j * k - r * i),
-                     2 * (i * k - r * j), 2 * (j * k + r * i), 1 - 2 * (i * i + j * j)], 1).view(-1, 3, 3)
+    R = _rotations(torch.nn.functional.normalize(out["quats"], dim=1))
     step = torch.einsum("nij,nj->ni", R, torch.exp(out["log_scales"]) * normals[src, child])
     out["means"] = torch.where(sp[:, None], out["means"] + step, out["means"])
     out["log_scales"] = torch.where(sp[:, None], out["log_scales"] - math.log(np.float32(1.6)), out["log_scales"])
