@@ -27,7 +27,7 @@ struct Layout {
     size_t gkey[2], gval[2];
     size_t pairs, scan_lb, sort_lb[2];
     size_t ikey[2], ival[2];
-    size_t ranges, tile_order, grad2d, pix_count, contrib, contrib_words, total;
+    size_t ranges, tile_order, grad2d, pix_count, contrib, total;
     size_t sort_lb_rows, scan_lb_rows;
     size_t tile_cnt, col_lb, col_lb_rows;
     int tiles_x, tiles_y, tiles, key_passes, depth_passes, tile_passes, tile_digit_bits;
@@ -35,8 +35,8 @@ struct Layout {
     int row_passes;
 };
 
-// Warps of a render block: 4 threads per tile row.
-int render_warps(int tile_h) { return (4 * tile_h + 31) / 32; }
+// 8x8-pixel sub-blocks of a tile: the render kernels' unit of contribution bits.
+int tile_subs(const gs_raster_config* c) { return (c->tile_w / 8) * (c->tile_h / 8); }
 
 bool valid_cfg(const gs_raster_config* c) {
     if (!c) return false;
@@ -111,10 +111,11 @@ bool make_layout(int n, int W, int H, uint64_t cap, const gs_raster_config* cfg,
     L->grad2d = take(nn * 12 * sizeof(float));
     // blended splats per pixel, written by the forward pass when gradients are limited
     L->pix_count = cfg->grad_limit > 0 ? take((size_t)W * H * sizeof(uint32_t)) : 0;
-    // contribution bits: per warp of a tile block, one bit per instance, set by the forward pass
-    // when some pixel of the warp blended that instance (the backward pass visits only those)
-    L->contrib_words = (cc + 31) / 32 + 2;
-    L->contrib = take((size_t)render_warps(cfg->tile_h) * L->contrib_words * sizeof(uint32_t));
+    // contribution bits: per sub-block of a tile, one bit per instance, written by the forward
+    // pass: whether some pixel of the sub-block blended that instance (the backward pass visits
+    // only those).  Tile t's words start at floor(start / 32) + t (start: its range), so no two
+    // tiles share a word; the words of a tile's sub-blocks are interleaved.
+    L->contrib = take((size_t)tile_subs(cfg) * (cc / 32 + L->tiles + 1) * sizeof(uint32_t));
     L->total = off;
     return true;
 }
@@ -618,7 +619,6 @@ gs_status bin_sort_impl(const FrameSet<MAXF>& fs, cudaStream_t s) {
 template <int MAXF>
 gs_status render_forward_impl(const FrameSet<MAXF>& fs, const float* bg, float* const* out_rgb,
                               float* const* out_T, uint32_t* const* out_last, cudaStream_t s) {
-    ClearArgs clr[MAXF];
     Multi<RenderFwdArgs, MAXF> m;
     m.frames = fs.count;
     for (int v = 0; v < fs.count; ++v) {
@@ -630,7 +630,6 @@ gs_status render_forward_impl(const FrameSet<MAXF>& fs, const float* bg, float* 
         a.cam = cam_k(f, L);
         a.cfg = cfg_k(f->cfg);
         for (int k = 0; k < 3; ++k) a.bg[k] = bg[3 * v + k];
-        a.batch = f->cfg.batch_depth;
         a.ranges = at<uint32_t>(ws, L.ranges);
         a.vals = at<uint32_t>(ws, vals_sorted_off(L));
         a.xy = at<float4>(ws, L.xy);
@@ -643,14 +642,8 @@ gs_status render_forward_impl(const FrameSet<MAXF>& fs, const float* bg, float* 
         a.capacity = f->capacity;
         a.status = &control_of(fs, v)->status;
         a.contrib = at<uint32_t>(ws, L.contrib);
-        a.contrib_words = (uint32_t)L.contrib_words;
         a.order = at<uint32_t>(ws, L.tile_order);
-        clr[v] = ClearArgs{};
-        clr[v].ptr[0] = a.contrib;
-        clr[v].words[0] = (unsigned long long)render_warps(f->cfg.tile_h) * L.contrib_words;
     }
-    gs_status st = clear_regions(fs, clr, s);
-    if (st != GS_OK) return st;
     return ok(launch_render_forward(m, s));
 }
 
@@ -675,7 +668,6 @@ gs_status render_backward_tiles_impl(const FrameSet<MAXF>& fs, const float* bg, 
         a.cam = cam_k(f, L);
         a.cfg = cfg_k(f->cfg);
         for (int k = 0; k < 3; ++k) a.bg[k] = bg[3 * v + k];
-        a.batch = f->cfg.batch_depth;
         a.ranges = at<uint32_t>(ws, L.ranges);
         a.vals = at<uint32_t>(ws, vals_sorted_off(L));
         a.xy = at<float4>(ws, L.xy);
@@ -690,7 +682,6 @@ gs_status render_backward_tiles_impl(const FrameSet<MAXF>& fs, const float* bg, 
         a.capacity = f->capacity;
         a.status = st;
         a.contrib = at<uint32_t>(ws, L.contrib);
-        a.contrib_words = (uint32_t)L.contrib_words;
         a.order = at<uint32_t>(ws, L.tile_order);
     }
     gs_status st = clear_regions(fs, clr, s);

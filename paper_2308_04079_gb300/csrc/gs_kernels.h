@@ -44,7 +44,7 @@ constexpr int kPairChunk = 2048;
 // Instance emission: 256 threads, one warp per 32 segment records.
 constexpr int kEmitThreads = 256;
 
-// Render: one block per tile, 4 threads per tile row, each owning tile_w / 4 pixels.
+// Render: one warp per block; groups of lanes own 8x8-pixel sub-blocks of the tiles (render.cu).
 
 // Batches: one launch per stage serves up to kMaxFrames frames (views of one scene, or of
 // several scenes).  A kernel receives the argument blocks of all its frames by value; frame f
@@ -270,7 +270,6 @@ struct RenderFwdArgs {
     CamK cam;
     CfgK cfg;
     float bg[3];
-    int batch;
     const uint32_t* ranges;
     const uint32_t* vals;
     const float4* xy;
@@ -282,8 +281,7 @@ struct RenderFwdArgs {
     uint32_t* out_count;       // nullable: blended splats per pixel (for cfg.grad_limit)
     unsigned long long capacity;   // instance capacity (GS_DEBUG range checks)
     gs_device_status* status;
-    uint32_t* contrib;         // per warp of a tile block: bit i set when the warp blended instance i (zeroed)
-    uint32_t contrib_words;    // words per warp
+    uint32_t* contrib;         // contribution bits per sub-block (see the workspace layout)
     const uint32_t* order;     // [tiles] the tile of each block (k_tile_order)
 };
 
@@ -292,7 +290,6 @@ struct RenderBwdArgs {
     CamK cam;
     CfgK cfg;
     float bg[3];
-    int batch;
     const uint32_t* ranges;
     const uint32_t* vals;
     const float4* xy;
@@ -307,7 +304,6 @@ struct RenderBwdArgs {
     unsigned long long capacity;   // instance capacity (GS_DEBUG range checks)
     gs_device_status* status;
     const uint32_t* contrib;   // the forward pass's contribution bits (see RenderFwdArgs)
-    uint32_t contrib_words;
     const uint32_t* order;     // [tiles] the tile of each block (k_tile_order)
 };
 

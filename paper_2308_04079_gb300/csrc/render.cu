@@ -1,26 +1,31 @@
 // render.cu -- per-tile blending (Algorithm 2, BlendInOrder) and its backward pass (Sec. 6).
 //
-// One thread block per tile; TPR = 4 threads per tile row, each owning PX = tile_w / TPR pixels
-// of that row (columns c, c + TPR, ...).  The block stages batches of the tile's depth-sorted Gaussians in
-// shared memory; a staged splat carries its offset from the tile's first pixel centre, the
-// Cholesky factor of its conic pre-scaled to log2 units, log2 of its opacity and its skip
-// threshold (see Staged), so that for a pixel at offset d:
+// A tile is made of 8x8-pixel sub-blocks (four in a 16x16 tile, two in 16x8, one in 8x8).  A group
+// of 8, 16 or 32 lanes of one warp owns a sub-block, each lane 8, 4 or 2 pixels of one row; a warp
+// (one per block) holds 4, 2 or 1 groups and no two warps wait on one another.  A warp stages the
+// next 32 Gaussians of its tile's depth-sorted list in shared memory (its tiles', when a tile has
+// fewer sub-blocks than the warp has groups) and each group then walks only the staged splats of
+// its own 32-bit word: in the forward those that can reach its sub-block, in the backward those
+// it blended.  The groups of a warp run through different splats in the same instructions, so the
+// per-splat work (loads, row setup, reduction) is shared by up to four splats.  Arithmetic on
+// pixel pairs is packed (f32x2).  What bounds the kernels is the issue slots and the latency of
+// few warps, not memory (profiles of the earlier one-warp-per-half-tile kernels: 77 % of the issue
+// slots at 59 % blended lanes per visited splat; 8x8 sub-blocks: 70 %).
+// A staged splat carries its offset from the tile's first pixel centre, the Cholesky factor of
+// its conic pre-scaled to log2 units and log2 of its opacity (Entry), so that for a pixel at
+// offset d:
 //   p = l11' dx + l21' dy, q = l22' dy, s = p^2 + q^2 = -log2(e) power,  o exp(power) = 2^(lo - s)
 // and "alpha < 1/255" is the single comparison s > thr with thr = lo - log2(1/255).  Pixels of
-// one row share dy, q and q^2, and p advances by TPR l11' from one owned pixel to the next, so a
-// skipped (pixel, splat) pair costs three instructions and no exp.
+// one row share dy, q and q^2; p is evaluated as that of one of the first four columns plus a
+// multiple of the step of four columns.
 //
 // Forward (eq. front-to-back, App. C): a = min(0.99, o exp(power)); skip a < 1/255; stop before
-//   T (1 - a) < 1e-4; C += a T c; T *= 1 - a.  The tile stops as soon as all its pixels are done
-//   (checked once per batch with __syncthreads_count).  Writes C + T bg, T and the 1-based list
-//   position of the last blended Gaussian.  The staging thread of a splat also computes, per
-//   warp (a band of 8 tile rows), whether the splat can reach alpha_min anywhere in the band
-//   (band_mask), and a warp skips the splats that cannot; for every 32 splats a warp ORs into
-//   its contribution bits (one bit per instance of the frame) those that some pixel of the
-//   warp blended.
-// Backward: the tile's list is walked back to front from the largest last position in the tile,
-//   each warp visiting only the splats its contribution bits name (it blends exactly the
-//   forward's pairs); each pixel only processes positions below its own last position, recovers
+//   T (1 - a) < 1e-4; C += a T c; T *= 1 - a.  A pixel that stopped has the sign bit of T set; a
+//   group stops when all its pixels have.  Writes C + T bg, T and the 1-based list position of the
+//   last blended Gaussian, and per sub-block one contribution word per 32 positions: the splats
+//   some pixel of the sub-block blended.
+// Backward: each group walks the splats its contribution words name back to front (it blends
+//   exactly the forward's pairs); each pixel only processes positions below its own last position, recovers
 //   T_i = T_{i+1} / (1 - a_i) from the stored final T, and keeps R . dL/dC, the projection of
 //   the colour behind the current Gaussian (normalised by the transmittance in front of it; R
 //   starts at bg) on the pixel's dL/dC, which is all the recurrence needs:
@@ -33,11 +38,9 @@
 //   In pixel coordinates the three entries of dL/dSigma' of an elongated splat are all dominated
 //   by its minor axis and their major-axis part, which the scale along the long axis needs, is
 //   lost to cancellation in fp32 sums over many pixels; in the whitened frame every direction of
-//   the splat has the same scale.  A thread sums its pixels' terms (mean, Sigma', opacity,
-//   colour); when more than kDirectLanes (24) lanes of a warp contributed, the warp sums its
-//   lanes with a transposed reduce-scatter (warp_reduce9) and nine lanes add the nine totals
-//   with one atomic instruction each, otherwise every contributing lane adds its own sums (two
-//   float4 atomics and one scalar).
+//   the splat has the same scale.  q being the row's, a lane sums dL/dpower with 1, p and p^2 over
+//   its pixels and multiplies by q and q^2 once; the nine sums of a group's lanes are reduced by a
+//   transposed reduce-scatter and every lane adds the one or two totals it holds.
 //
 // Limited-BW (cfg.grad_limit = N > 0, the ablation of Sec. 7.3): the forward pass also records
 // the number of blended splats of every pixel (COUNT); the backward pass (LIMIT) keeps the
@@ -45,13 +48,15 @@
 // gradient terms of the first (count - N) blended splats it meets from the back.
 //
 // The forward and the backward evaluate a (pixel, splat) pair with the same staging and the same
-// operation sequence (stage_splat, splat_row, splat_s), so their skip and clamp decisions agree
-// bit for bit.
+// operation sequence (stage_splat, splat_row), whatever the pixels per lane, so their skip and
+// clamp decisions agree bit for bit.
 //
-// Block order: block b of a frame renders tile order[b], the frame's tiles by decreasing list
+// Block order: warps take the tiles in the order of order[], the frame's tiles by decreasing list
 // length (k_tile_order, run at the end of the binning stage).  The work of a tile grows with its
 // list and varies by a factor of several across a frame; blocks start roughly in index order, so
 // in row-major order the longest tiles (the frame's centre) could start late and finish alone.
+#include <type_traits>
+
 #include "gs_device.cuh"
 #include "gs_kernels.h"
 
@@ -65,9 +70,10 @@ constexpr float kScaleLog2 = 0.84932180028801907f;
 constexpr float kUnscale = 1.1774100225154747f;
 // (1/2) / kScaleLog2^2 = ln 2: scaled (p, q)(p, q)^T sums to K = (1/2) sum dL/dpower (p, q)(p, q)^T.
 constexpr float kLn2 = 0.69314718055994531f;
-// At most this many contributing lanes add their own sums instead of a warp reduction (measured
-// on the 3M-Gaussian 1080p frame: 24 beats 6, 12, 16, 20 and 32).
-constexpr int kDirectLanes = 24;
+// Side of a sub-block in pixels: the unit of culling, contribution bits and lane groups.
+constexpr int kSub = 8;
+// Magnitude of dL/dC, colour or conic from which pixels' products are kept apart (backward_unit).
+constexpr float kWild = 1.0e30f;
 
 struct Staged {
     float4 a;   // (ox, oy, thr, lo): tile-relative offset, skip threshold, log2(opacity)
@@ -103,92 +109,222 @@ __device__ __forceinline__ float rect_min_s(const Staged& st, float xa, float xb
     return m;
 }
 
-// Warps of a render block (bit w) whose band of tile rows [w rows_per_warp, (w + 1) rows_per_warp)
-// holds a point where the staged splat reaches alpha_min: the minimum of its quadratic form over
-// the band's rectangle (continuous, so it covers every pixel centre) within a small margin of the
-// threshold.  A cleared bit proves no pixel of that warp blends the splat.
-__device__ __forceinline__ uint32_t band_mask(const Staged& st, int tile_w, int tile_h, int rows_per_warp) {
+// Whether the staged splat can reach alpha_min at a point of an 8x8 sub-block whose first pixel
+// centre is at offset (xa, ya) from the splat: the minimum of its quadratic form over the
+// sub-block's rectangle (continuous, so it covers every pixel centre) within a small margin of the
+// threshold.  False proves no pixel of the sub-block blends the splat.
+__device__ __forceinline__ bool sub_reach(const Staged& st, float xa, float ya) {
     const float thr = st.a.z;
-    if (!(thr > 0.f)) return 0u;
+    if (!(thr > 0.f)) return false;
     const float lim = fmaf(thr, 1.0009765625f, 0.0009765625f);   // thr (1 + 2^-10) + 2^-10
-    uint32_t m = 0;
-    for (int w = 0; w * rows_per_warp < tile_h; ++w) {
-        const float ya = st.a.y + (float)(w * rows_per_warp), yb = ya + (float)(rows_per_warp - 1);
-        if (rect_min_s(st, st.a.x, st.a.x + (float)(tile_w - 1), ya, yb) <= lim) m |= 1u << w;
+    return rect_min_s(st, xa, xa + (float)(kSub - 1), ya, ya + (float)(kSub - 1)) <= lim;
+}
+
+// ---- pairs of fp32 values in one 64-bit register (PTX f32x2: two IEEE round-to-nearest
+// operations in one issue slot) -------------------------------------------------------------
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float sum2(f32x2 v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
+    return lo + hi;
+}
+
+// The part of the frame a lane works on.  Groups (sub-blocks) are numbered tile by tile in the
+// render order; a warp takes GW consecutive groups.  With more groups in a warp than sub-blocks
+// in a tile, the warp holds several tiles, each staged by its own lanes.
+template <int PX, int SUBS>
+struct Lanes {
+    static constexpr int LPR = kSub / PX;                    // lanes per pixel row of a sub-block
+    static constexpr int GL = kSub * LPR;                    // lanes of a group
+    static constexpr int GW = 32 / GL;                       // groups of a warp
+    static constexpr int SX = SUBS >= 2 ? 2 : 1;             // sub-blocks per tile row
+    static constexpr int NS = SUBS < GW ? SUBS : GW;         // sub-blocks of one tile in a warp
+    static constexpr int TPW = GW / NS;                      // tiles in a warp
+    static constexpr int SL = 32 / TPW;                      // lanes staging one tile
+    static constexpr int ROUNDS = 32 / SL;                   // splats a lane stages per window
+    static constexpr int PAIRS = PX / 2;
+    // fetch the next window's splats while one is blended (registers allow it with one splat per lane)
+    static constexpr bool AHEAD = ROUNDS == 1 && PX < 8;
+    // blend every splat with care (Entry): with few pixels per lane that costs less than a second path
+    static constexpr bool ONE_PATH = PX == 2;
+    int lane, group, slot, tl, sub, sx, sy, row, col;
+    uint32_t index;                                          // of the tile in the render order
+    __device__ __forceinline__ explicit Lanes(uint32_t unit) {
+        lane = threadIdx.x & 31;
+        group = lane / GL;
+        slot = lane / SL;
+        tl = lane % SL;
+        const uint32_t gid = unit * GW + (uint32_t)group;
+        index = gid / SUBS;
+        sub = (int)(gid % SUBS);
+        sx = sub % SX;
+        sy = sub / SX;
+        row = (lane % GL) / LPR;
+        col = (lane % LPR) * PX;                             // first owned column in the sub-block
     }
-    return m;
+    // Column of the i-th owned pixel in the tile is 8 sx + col + i; its offset is evaluated as
+    // that of column c0 = (col + i) & 3 plus j() steps of four columns.
+    __device__ __forceinline__ float j(int i) const { return (float)(2 * sx + (PX == 8 ? i / 4 : col / 4)); }
+    __device__ __forceinline__ float c0(int i) const { return PX == 2 ? (float)((col & 3) + i) : (float)(i & 3); }
+    // Sub-blocks of this warp's tiles: the s-th of NS is sub0() + s.
+    __device__ __forceinline__ int sub0() const { return sub - (group % NS); }
+};
+
+// A staged splat in shared memory: what the packed arithmetic broadcasts is stored twice, so that a
+// 16-byte load yields register pairs (20 move instructions fewer per splat and warp).  Bit 31 of
+// `id` marks a splat whose pairs need care: its alpha can reach alpha_max, its conic is not finite
+// (a degenerate splat without dilation) or its colour could overflow a product.
+struct __align__(16) Entry {
+    f32x2 ox, oy;         // offset of the tile's first pixel centre from the mean
+    f32x2 l11, l21;       // scaled Cholesky factor of the conic
+    f32x2 l22, lo;        // lo = log2(opacity)
+    f32x2 r, g;           // colour
+    f32x2 b;
+    float ko;             // 1 / opacity
+    uint32_t id;          // Gaussian | care << 31
+};
+
+__device__ __forceinline__ Entry entry_of(const Staged& st, float4 col, uint32_t gid, float lo_care) {
+    Entry e;
+    e.ox = pack2(st.a.x, st.a.x);
+    e.oy = pack2(st.a.y, st.a.y);
+    e.l11 = pack2(st.b.x, st.b.x);
+    e.l21 = pack2(st.b.y, st.b.y);
+    e.l22 = pack2(st.b.z, st.b.z);
+    e.lo = pack2(st.a.w, st.a.w);
+    e.r = pack2(col.x, col.x);
+    e.g = pack2(col.y, col.y);
+    e.b = pack2(col.z, col.z);
+    e.ko = st.b.w;
+    const bool care = !(st.a.w <= lo_care) || !(fabsf(st.b.x) + fabsf(st.b.y) + fabsf(st.b.z) < kWild) ||
+                      !(col.x + col.y + col.z < kWild);   // colours are clamped at 0
+    e.id = gid | (care ? 0x80000000u : 0u);
+    return e;
 }
 
-// 32 bits of a contribution bit array ending at bit `hi` (bit 31 = bit hi, bit 0 = bit hi - 31;
-// bits below 0 read as 0).
-__device__ __forceinline__ uint32_t bits_window(const uint32_t* w, uint32_t hi) {
-    const uint32_t word = hi >> 5, sh = hi & 31u;
-    const uint32_t top = w[word] << (31u - sh);
-    const uint32_t low = (sh < 31u && word > 0) ? (w[word - 1] >> (sh + 1u)) : 0u;
-    return top | low;
-}
-
-// Sum over the warp of the 9 accumulators v[0..8] by a transposed reduce-scatter: each round
-// halves the values a lane keeps (it sends the half its partner keeps and adds the half it
-// receives), 12 shuffles instead of 45.  Afterwards the total of accumulator slot(lane) is in
-// the even lanes of each pair (slot < 0: padding); see reduce_slot.
-__device__ __forceinline__ float warp_reduce9(const float (&v)[9], int lane) {
-    float a[5];
-    const bool h16 = lane & 16;
+// What a lane fetches of a splat it stages.
+struct Fetched {
+    float4 xy, conic, rgb;
+    uint32_t id;
+};
+// The Gaussians a lane stages of a window: positions first, first + SL, ... of its tile's list,
+// those below `len`.
+template <int ROUNDS, int SL>
+__device__ __forceinline__ void fetch_ids(uint32_t (&id)[ROUNDS], const uint32_t* vals, uint32_t first, uint32_t len) {
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {   // lanes 0-15 keep v[0..4], lanes 16-31 keep v[5..8] (+ padding)
-        const float lo = v[i], hi = i < 4 ? v[5 + i] : 0.f;
-        a[i] = (h16 ? hi : lo) + __shfl_xor_sync(0xffffffffu, h16 ? lo : hi, 16);
+    for (int r = 0; r < ROUNDS; ++r) id[r] = first + (uint32_t)(r * SL) < len ? vals[first + (uint32_t)(r * SL)] : 0u;
+}
+template <typename A>
+__device__ __forceinline__ void fetch_splat(Fetched& f, uint32_t g, const A& a) {
+    if (g >= (uint32_t)a.n) {   // only reachable after a timed-out sort
+        debug_fail(a.status);
+        g = 0;
     }
-    float b[3];
-    const bool h8 = lane & 8;
+    f.id = g;
+    f.xy = a.xy[g];
+    f.conic = a.conic_opacity[g];
+    f.rgb = a.rgb[g];
+}
+
+// log2 of an opacity whose alpha stays below alpha_max whatever the rounding of 2^x.
+__device__ __forceinline__ float log2_care(float alpha_max) { return __log2f(alpha_max) - 1.0e-5f; }
+
+// A splat along the lane's pixel row: p at the pairs of columns (0, 1) and (2, 3) of the
+// four-column step, its step dp, q and q^2 (in both halves).
+struct RowPairs {
+    f32x2 p0[2], dp, q, qq;
+};
+template <int PX, int SUBS>
+__device__ __forceinline__ RowPairs splat_row(const Lanes<PX, SUBS>& ln, const Entry& e, f32x2 ly) {
+    RowPairs r;
+    const f32x2 dy = add2(ly, e.oy);
+    r.q = mul2(e.l22, dy);
+    r.qq = mul2(r.q, r.q);
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {   // keep a[0..2] or a[3..4] (+ padding)
-        const float lo = a[i], hi = i < 2 ? a[3 + i] : 0.f;
-        b[i] = (h8 ? hi : lo) + __shfl_xor_sync(0xffffffffu, h8 ? lo : hi, 8);
+    for (int h = 0; h < (PX == 2 ? 1 : 2); ++h) {
+        const f32x2 dx0 = add2(pack2(ln.c0(2 * h), ln.c0(2 * h + 1)), e.ox);
+        r.p0[h] = fma2(e.l21, dy, mul2(e.l11, dx0));
     }
-    float c[2];
-    const bool h4 = lane & 4;
+    r.dp = mul2(pack2(4.0f, 4.0f), e.l11);
+    return r;
+}
+__device__ __forceinline__ float low(f32x2 v) {
+    float lo, hi;
+    unpack2(v, lo, hi);
+    return lo;
+}
+
+// Sum over the lanes of a group of 9 values by a transposed reduce-scatter: each round halves the
+// values a lane keeps (it sends the half its partner keeps and adds the half it receives).  The
+// totals of slots [first, first + n) of reduce_slots are left in out[0..1].
+template <int GL>
+__device__ __forceinline__ void group_reduce9(const float (&v)[9], int lane, float (&out)[2]) {
+    float a[9];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {   // keep b[0..1] or b[2] (+ padding)
-        const float lo = b[i], hi = i < 1 ? b[2] : 0.f;
-        c[i] = (h4 ? hi : lo) + __shfl_xor_sync(0xffffffffu, h4 ? lo : hi, 4);
+    for (int i = 0; i < 9; ++i) a[i] = v[i];
+    int n = 9;
+#pragma unroll
+    for (int m = GL / 2; m > 0; m >>= 1) {
+        const bool hi = lane & m;
+        const int half = (n + 1) / 2;
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            if (i >= half) continue;
+            if (half + i < n) {
+                const float keep = hi ? a[half + i] : a[i], send = hi ? a[i] : a[half + i];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+            } else {   // the odd value: both sides keep its sum
+                a[i] += __shfl_xor_sync(0xffffffffu, a[i], m);
+            }
+        }
+        n = half;
     }
-    const bool h2 = lane & 2;
-    float d = (h2 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h2 ? c[0] : c[1], 2);
-    d += __shfl_xor_sync(0xffffffffu, d, 1);
-    return d;
+    out[0] = a[0];
+    out[1] = a[1];
 }
 
-// Accumulator slot whose warp total warp_reduce9 leaves in `lane` (-1: padding).
-__device__ __forceinline__ int reduce_slot(int lane) {
-    const int base = (lane & 16) ? 5 : 0;   // values kept after the first round
-    int l3[3];
-    if (lane & 8) { l3[0] = base + 3; l3[1] = base + 4; l3[2] = -1; }
-    else { l3[0] = base; l3[1] = base + 1; l3[2] = base + 2; }
-    int l2[2];
-    if (lane & 4) { l2[0] = l3[2]; l2[1] = -1; }
-    else { l2[0] = l3[0]; l2[1] = l3[1]; }
-    const int slot = (lane & 2) ? l2[1] : l2[0];
-    return slot > 8 ? -1 : slot;
-}
-
-// Per (thread row, splat): p at the thread's first pixel, its step to the next owned pixel
-// (`step` columns to the right), q, q^2.
-__device__ __forceinline__ void splat_row(const Staged& s, float lyf, float c0f, float step, float& p0, float& dp,
-                                          float& q, float& qq) {
-    const float dy = __fadd_rn(lyf, s.a.y);
-    const float dx0 = __fadd_rn(c0f, s.a.x);
-    q = __fmul_rn(s.b.z, dy);
-    qq = __fmul_rn(q, q);
-    p0 = __fmaf_rn(s.b.y, dy, __fmul_rn(s.b.x, dx0));
-    dp = __fmul_rn(step, s.b.x);
-}
-
-// s = p^2 + q^2 at the thread's j-th pixel.
-__device__ __forceinline__ float splat_s(float p0, float dp, float qq, int j, float& p) {
-    p = __fmaf_rn((float)j, dp, p0);
-    return __fmaf_rn(p, p, qq);
+// Slots [first, first + n) whose totals group_reduce9 leaves in this lane (n <= 2; a slot is
+// owned by one lane of the group).
+template <int GL>
+__device__ __forceinline__ void reduce_slots(int lane, int& first, int& n) {
+    first = 0;
+    n = 9;
+    int len = 9;
+#pragma unroll
+    for (int m = GL / 2; m > 0; m >>= 1) {
+        const int half = (len + 1) / 2;
+        const bool odd_tail = len == 1;   // one value left: both sides hold it, the lower lane owns it
+        if (lane & m) {
+            first += half;
+            n = odd_tail ? 0 : (n > half ? n - half : 0);
+        } else {
+            n = n < half ? n : half;
+        }
+        len = half;
+    }
 }
 
 constexpr int kOrderThreads = 1024;
@@ -253,384 +389,560 @@ __global__ void __launch_bounds__(kOrderThreads) k_tile_order(const __grid_const
     }
 }
 
-// Forward pass of the tile order[block_slot] of a frame with ntiles tiles.
-template <int PX, int TPR, bool COUNT>
-__device__ __forceinline__ void forward_tile(const RenderFwdArgs& a, uint32_t block_slot, uint32_t ntiles) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Staged* s_sp = reinterpret_cast<Staged*>(smem_raw);
-    float4* s_rgb = reinterpret_cast<float4*>(smem_raw + sizeof(Staged) * a.batch);
-    uint32_t* s_band = reinterpret_cast<uint32_t*>(smem_raw + (sizeof(Staged) + sizeof(float4)) * a.batch);
-    const CamK& c = a.cam;
-    const uint32_t tile_id = a.order[block_slot];
-    if (tile_id >= ntiles) {   // an order not written by gs_bin_sort
-        if (threadIdx.x == 0) debug_fail(a.status);
-        return;
-    }
-    const int tile = (int)tile_id;
-    const int tx = tile % c.tiles_x, ty = tile / c.tiles_x;
-    const int nthreads = blockDim.x;
-    const int ly = threadIdx.x / TPR, c0 = threadIdx.x % TPR;   // TPR threads per tile row
-    const int x0 = tx * c.tile_w, y0 = ty * c.tile_h;
-    const int py = y0 + ly;
-    const float lyf = (float)ly, c0f = (float)c0;
-    const int warp = threadIdx.x >> 5;
-    const uint32_t start = a.ranges[2 * tile];
-    uint32_t end = a.ranges[2 * tile + 1];
-    if (GS_DEBUG && (end < start || end > a.capacity)) {   // a range outside the instance lists
-        if (threadIdx.x == 0) debug_fail(a.status);
-        end = start;
-    }
-    const int lane = threadIdx.x & 31;
-    uint32_t* const wbits = a.contrib + (size_t)(threadIdx.x >> 5) * a.contrib_words;
-    const float amax = a.cfg.alpha_max, tmin = a.cfg.T_min;
-    const float log2_amin = __log2f(a.cfg.alpha_min);
-    // what the loops read, in registers
-    const int batch = a.batch, n = a.n, tile_w = c.tile_w, tile_h = c.tile_h;
-    const uint32_t* const vals = a.vals;
-    const float4* const xy = a.xy;
-    const float4* const conic = a.conic_opacity;
-    const float4* const rgb = a.rgb;
+// The decisions of a pixel pair against one splat: alpha >= 1/255 (s <= thr), and stop before T (1 - alpha)
+// < T_min.  A pixel that blends takes `te` and its `last`; one that stops gets its sign bit set.
+// Returns the blend weights alpha T (0 when not blended); a0, a1: the bits of the blended alphas.
+// Written in PTX for the dual-output comparison and in-place selects.  `on`
+// false skips the pair.
+__device__ __forceinline__ f32x2 blend_pair(f32x2 s, float thr, f32x2 al, f32x2 te, float tmin, uint32_t pos, bool on,
+                                            f32x2& T, uint32_t& last0, uint32_t& last1, uint32_t& a0, uint32_t& a1) {
+    f32x2 w;
+    asm("{\n\t.reg .pred h0, h1, k0, k1, z0, z1;\n\t.reg .f32 s0, s1, t0, t1, e0, e1, x0, x1;\n\t.reg .b64 A;\n\t"
+            "mov.b64 {s0, s1}, %6;\n\tmov.b64 {t0, t1}, %1;\n\tmov.b64 {e0, e1}, %9;\n\tmov.b64 {x0, x1}, %8;\n\t"
+            "setp.ne.s32 h0, %12, 0;\n\tsetp.leu.and.f32 h1, s1, %7, h0;\n\tsetp.leu.and.f32 h0, s0, %7, h0;\n\t"
+            "setp.geu.and.f32 k0|z0, e0, %10, h0;\n\tsetp.geu.and.f32 k1|z1, e1, %10, h1;\n\t"
+            "selp.f32 x0, x0, 0f00000000, k0;\n\tselp.f32 x1, x1, 0f00000000, k1;\n\t"
+            "mov.b64 A, {x0, x1};\n\tmul.rn.f32x2 %0, A, %1;\n\t"
+            "selp.f32 t0, e0, t0, k0;\n\tselp.f32 t1, e1, t1, k1;\n\t"
+            "@z0 or.b32 t0, t0, 0x80000000;\n\t@z1 or.b32 t1, t1, 0x80000000;\n\t"
+            "mov.b64 %1, {t0, t1};\n\t@k0 mov.u32 %2, %11;\n\t@k1 mov.u32 %3, %11;\n\t"
+            "mov.b32 %4, x0;\n\tmov.b32 %5, x1;\n\t}"
+            : "=l"(w), "+l"(T), "+r"(last0), "+r"(last1), "=r"(a0), "=r"(a1)
+            : "l"(s), "f"(thr), "l"(al), "l"(te), "f"(tmin), "r"(pos), "r"((int)on));
+    return w;
+}
 
-    float T[PX], Cr[PX], Cg[PX], Cb[PX];
-    uint32_t last[PX], nblended[PX];
-    bool done[PX];
-    int ndone = 0;
-#pragma unroll
-    for (int j = 0; j < PX; ++j) {
-        T[j] = 1.0f;
-        Cr[j] = Cg[j] = Cb[j] = 0.f;
-        last[j] = 0;
-        nblended[j] = 0;
-        done[j] = !(x0 + c0 + TPR * j < c.W && py < c.H);
-        ndone += done[j];
-    }
-    for (uint32_t b = start; b < end; b += batch) {
-        if (__syncthreads_count(ndone == PX) == nthreads) break;
-        const int nb = (int)min((uint32_t)batch, end - b);
-        for (int k = threadIdx.x; k < nb; k += nthreads) {
-            uint32_t g = vals[b + k];
-            if (g >= (uint32_t)n) {   // only reachable after a timed-out sort
-                debug_fail(a.status);
-                g = 0;
-            }
-            Staged st;
-            stage_splat(xy[g], conic[g], x0, y0, log2_amin, st);
-            s_sp[k] = st;
-            s_rgb[k] = rgb[g];
-            s_band[k] = band_mask(st, tile_w, tile_h, 32 / TPR);
+// Forward pass of the groups of one warp (`unit`) of a frame with ntiles tiles.
+template <int PX, int SUBS, bool COUNT>
+__device__ __forceinline__ void forward_unit(const RenderFwdArgs& a, uint32_t unit, uint32_t ntiles) {
+    using LN = Lanes<PX, SUBS>;
+    constexpr int U = PX == 2 ? 4 : 2;
+    __shared__ Entry s_e[LN::TPW][32];
+    const LN ln(unit);
+    const CamK& c = a.cam;
+    const uint32_t full = 0xffffffffu;
+    uint32_t tile = ln.index < ntiles ? a.order[ln.index] : 0u;
+    const bool live = ln.index < ntiles && tile < ntiles;
+    if (ln.index < ntiles && !live && ln.tl == 0) debug_fail(a.status);   // an order not written by gs_bin_sort
+    if (!live) tile = 0;
+    const int tx = (int)tile % c.tiles_x, ty = (int)tile / c.tiles_x;
+    const int x0 = tx * (kSub * LN::SX), y0 = ty * c.tile_h;
+    const int ly = kSub * ln.sy + ln.row, py = y0 + ly, px0 = x0 + kSub * ln.sx + ln.col;
+    const f32x2 lyf = pack2((float)ly, (float)ly);
+    uint32_t start = 0, len = 0;
+    if (live) {
+        const uint2 r = *reinterpret_cast<const uint2*>(a.ranges + 2 * tile);
+        start = r.x;
+        len = r.y - r.x;
+        if (GS_DEBUG && (r.y < r.x || r.y > a.capacity)) {   // a range outside the instance lists
+            if (ln.tl == 0) debug_fail(a.status);
+            len = 0;
         }
-        __syncthreads();
-        // 32 splats at a time: the warp's contribution bits for them are one word
-        for (int k0 = 0; k0 < nb; k0 += 32) {
-            uint32_t mb = 0;   // bit k - k0: some pixel of this thread blended splat k
-            if (ndone < PX) {
-                const int k1 = min(k0 + 32, nb);
-#pragma unroll 2   // lets the next splat's row setup overlap this one's blend (forward 0.340 -> 0.333 ms)
-                for (int k = k0; k < k1; ++k) {
-                    if (!((s_band[k] >> warp) & 1u)) continue;           // no pixel of this warp reaches alpha_min
-                    const Staged st = s_sp[k];
-                    float p0, dp, q, qq;
-                    splat_row(st, lyf, c0f, (float)TPR, p0, dp, q, qq);
-                    if (qq > st.a.z) continue;                         // s >= q^2: the whole row skips
+    }
+    uint32_t* const bits = a.contrib + (size_t)((start >> 5) + tile) * SUBS + ln.sub;
+    const float amax = a.cfg.alpha_max, tmin = a.cfg.T_min;
+    const float log2_amin = __log2f(a.cfg.alpha_min), lo_care = log2_care(amax);
+    const uint32_t* const vals = a.vals + start;
+    const f32x2 one = pack2(1.f, 1.f), neg = pack2(-1.f, -1.f);
+
+    // a pixel is done (stopped, or outside the image) when its T is negative
+    f32x2 T[LN::PAIRS], Cr[LN::PAIRS], Cg[LN::PAIRS], Cb[LN::PAIRS];
+    uint32_t last[PX], nblended[PX];
 #pragma unroll
-                    for (int j = 0; j < PX; ++j) {
-                        float p;
-                        const float s = splat_s(p0, dp, qq, j, p);
-                        if (done[j] || s > st.a.z) continue;           // alpha < 1/255: skip
-                        const float oG = hw_exp2(__fsub_rn(st.a.w, s));
-                        const float alpha = fminf(amax, oG);
-                        const float test = __fmul_rn(T[j], __fsub_rn(1.0f, alpha));
-                        if (test < tmin) {                             // stop before exceeding 0.9999
-                            done[j] = true;
-                            ++ndone;
-                            continue;
-                        }
-                        const float w = alpha * T[j];
-                        const float4 col = s_rgb[k];
-                        Cr[j] += w * col.x;
-                        Cg[j] += w * col.y;
-                        Cb[j] += w * col.z;
-                        T[j] = test;
-                        last[j] = b - start + (uint32_t)k + 1u;
-                        mb |= 1u << (k - k0);
-                        if (COUNT) ++nblended[j];
-                    }
-                    if (ndone == PX) break;
+    for (int i = 0; i < PX; ++i) last[i] = nblended[i] = 0;
+#pragma unroll
+    for (int i = 0; i < LN::PAIRS; ++i) {
+        const bool row_in = live && py < c.H;
+        T[i] = pack2(row_in && px0 + 2 * i < c.W ? 1.0f : -1.0f, row_in && px0 + 2 * i + 1 < c.W ? 1.0f : -1.0f);
+        Cr[i] = Cg[i] = Cb[i] = pack2(0.f, 0.f);
+    }
+
+    Fetched fetched;
+    uint32_t ids[LN::ROUNDS];
+    if (a.n > 0) {
+        fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, (uint32_t)ln.tl, len);
+        if (LN::AHEAD) {
+            fetch_splat(fetched, ids[0], a);
+            fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, 32u + (uint32_t)ln.tl, len);
+        }
+    }
+    const uint32_t gmask = LN::GL == 32 ? full : ((1u << (LN::GL & 31)) - 1u) << (ln.group * LN::GL & 31);
+    for (uint32_t base = 0;; base += 32) {
+        bool alive = false;
+#pragma unroll
+        for (int i = 0; i < LN::PAIRS; ++i) {
+            float t[2];
+            unpack2(T[i], t[0], t[1]);
+            alive |= t[0] > 0.f || t[1] > 0.f;
+        }
+        const uint32_t who = __ballot_sync(full, alive && base < len);
+        if (who == 0) break;
+        const bool active = (who & gmask) != 0;                // this group
+        // stage the next 32 splats of the tile; bit k of a group's word: splat base + k can
+        // reach its sub-block
+        uint32_t word = 0;
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < LN::ROUNDS; ++r) {
+            const int k = ln.tl + r * LN::SL;
+            uint32_t reach = 0;
+            if (base + (uint32_t)k < len) {
+                if (!LN::AHEAD) fetch_splat(fetched, ids[r], a);
+                Staged st;
+                stage_splat(fetched.xy, fetched.conic, x0, y0, log2_amin, st);
+                s_e[ln.slot][k] = entry_of(st, fetched.rgb, fetched.id, lo_care);
+                const int s0 = ln.sub0();
+#pragma unroll
+                for (int s = 0; s < LN::NS; ++s) {
+                    const int sx = (s0 + s) % LN::SX, sy = (s0 + s) / LN::SX;
+                    if (sub_reach(st, st.a.x + (float)(kSub * sx), st.a.y + (float)(kSub * sy))) reach |= 1u << s;
                 }
             }
-            mb = __reduce_or_sync(0xffffffffu, mb);
-            if (lane == 0 && mb) {   // instances b + k0 .. b + k0 + 31 of this warp's bit array
-                const uint32_t gi = b + (uint32_t)k0, sh = gi & 31u;
-                atomicOr(wbits + (gi >> 5), mb << sh);
-                if (sh) atomicOr(wbits + (gi >> 5) + 1, mb >> (32u - sh));
+#pragma unroll
+            for (int s = 0; s < LN::NS; ++s) {
+                uint32_t bal = __ballot_sync(full, (reach >> s) & 1u);
+                if (LN::SL < 32) bal = ((bal >> (ln.slot * LN::SL & 31)) & ((1u << (LN::SL & 31)) - 1u)) << (r * LN::SL & 31);
+                if (ln.group % LN::NS == s) word |= bal;
             }
-            if (__all_sync(0xffffffffu, ndone == PX)) break;
         }
+        if (!active) word = 0;
+        // in flight while this window is blended
+        if (LN::AHEAD) fetch_splat(fetched, ids[0], a);
+        fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, base + (LN::AHEAD ? 64u : 32u) + (uint32_t)ln.tl, len);
+        __syncwarp();
+        uint32_t mb = 0;   // bit k: a pixel of this lane blended splat base + k
+        while (word) {
+            // the next U splats of the group, front to back
+            Entry e[U];
+            uint32_t bit[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int k = word ? __ffs(word) - 1 : 0;
+                bit[u] = word & (0u - word);                   // 0: none left
+                word &= word - 1u;
+                e[u] = s_e[ln.slot][k];
+            }
+            auto blend = [&](auto care) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const RowPairs row = splat_row(ln, e[u], lyf);
+                    const float thr = __fsub_rn(low(e[u].lo), log2_amin);
+                    const bool on = bit[u] != 0 && !(low(row.qq) > thr);   // s >= q^2: else the whole row skips
+                    const uint32_t pos = base + 32u - (uint32_t)__clz((int)bit[u]);
+                    uint32_t any = 0;
+#pragma unroll
+                    for (int i = 0; i < LN::PAIRS; ++i) {
+                        const float jj = ln.j(2 * i);
+                        const f32x2 p = fma2(pack2(jj, jj), row.dp, row.p0[i & 1]);
+                        const f32x2 s = fma2(p, p, row.qq);
+                        const f32x2 x = fma2(s, neg, e[u].lo);     // lo - s
+                        float xv[2], al[2];
+                        unpack2(x, xv[0], xv[1]);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            al[h] = hw_exp2(xv[h]);
+                            if (decltype(care)::value) al[h] = fminf(amax, al[h]);
+                        }
+                        const f32x2 al2 = pack2(al[0], al[1]);
+                        const f32x2 te = mul2(T[i], fma2(al2, neg, one));   // T (1 - alpha)
+                        uint32_t a0, a1;
+                        const f32x2 w = blend_pair(s, thr, al2, te, tmin, pos, on, T[i], last[2 * i], last[2 * i + 1], a0, a1);
+                        any |= a0 | a1;
+                        if (COUNT) {
+                            nblended[2 * i] += a0 != 0;
+                            nblended[2 * i + 1] += a1 != 0;
+                        }
+                        Cr[i] = fma2(w, e[u].r, Cr[i]);
+                        Cg[i] = fma2(w, e[u].g, Cg[i]);
+                        Cb[i] = fma2(w, e[u].b, Cb[i]);
+                    }
+                    if (any) mb |= bit[u];
+                }
+            };
+            uint32_t flags = e[0].id;
+#pragma unroll
+            for (int u = 1; u < U; ++u) flags |= e[u].id;
+            if (LN::ONE_PATH || (int)flags < 0) blend(std::true_type{});
+            else blend(std::false_type{});
+        }
+#pragma unroll
+        for (int m = LN::GL / 2; m > 0; m >>= 1) mb |= __shfl_xor_sync(full, mb, m);
+        // every word the group walks is written: the backward pass reads no other
+        if (active && ln.lane % LN::GL == 0) bits[(size_t)(base >> 5) * SUBS] = mb;
     }
     const size_t P = (size_t)c.W * c.H;
 #pragma unroll
-    for (int j = 0; j < PX; ++j) {
-        const int px = x0 + c0 + TPR * j;
-        if (px < c.W && py < c.H) {
+    for (int i = 0; i < PX; ++i) {
+        const int px = px0 + i;
+        if (live && px < c.W && py < c.H) {
             const size_t p = (size_t)py * c.W + px;
-            a.out_rgb[p] = Cr[j] + T[j] * a.bg[0];
-            a.out_rgb[P + p] = Cg[j] + T[j] * a.bg[1];
-            a.out_rgb[2 * P + p] = Cb[j] + T[j] * a.bg[2];
-            a.out_T[p] = T[j];
-            a.out_last[p] = last[j];
-            if (COUNT) a.out_count[p] = nblended[j];
+            float r[2], g[2], b[2], tt[2];
+            unpack2(T[i / 2], tt[0], tt[1]);
+            unpack2(Cr[i / 2], r[0], r[1]);
+            unpack2(Cg[i / 2], g[0], g[1]);
+            unpack2(Cb[i / 2], b[0], b[1]);
+            const float t = fabsf(tt[i & 1]);
+            a.out_rgb[p] = r[i & 1] + t * a.bg[0];
+            a.out_rgb[P + p] = g[i & 1] + t * a.bg[1];
+            a.out_rgb[2 * P + p] = b[i & 1] + t * a.bg[2];
+            a.out_T[p] = t;
+            a.out_last[p] = last[i];
+            if (COUNT) a.out_count[p] = nblended[i];
         }
     }
 }
 
-// One block per tile.  A single frame reads its arguments straight from the parameter bank; a
+// One warp per block.  A single frame reads its arguments straight from the parameter bank; a
 // batch copies its frame's block of arguments into registers once (measured on four 1M-Gaussian
 // views: half the instructions of a shared-memory copy, whose compiled form executed the blend
 // loop's skipped pairs at the cost of blended ones).
-template <int PX, int TPR, int MAXF, bool COUNT>
-__global__ void __launch_bounds__(64, 1) k_render_forward_t(const __grid_constant__ Multi<RenderFwdArgs, MAXF> m) {
+template <int PX, int SUBS, int MAXF, bool COUNT>
+__global__ void __launch_bounds__(32, 16) k_render_forward_t(const __grid_constant__ Multi<RenderFwdArgs, MAXF> m) {
     if constexpr (MAXF == 1) {
-        forward_tile<PX, TPR, COUNT>(m.a[0], blockIdx.x, m.base[1]);
+        forward_unit<PX, SUBS, COUNT>(m.a[0], blockIdx.x, (uint32_t)(m.a[0].cam.tiles_x * m.a[0].cam.tiles_y));
     } else {
         const int f = find_frame<MAXF>(m.base, m.frames, blockIdx.x);
         const RenderFwdArgs a = m.a[f];
-        forward_tile<PX, TPR, COUNT>(a, blockIdx.x - m.base[f], m.base[f + 1] - m.base[f]);
+        forward_unit<PX, SUBS, COUNT>(a, blockIdx.x - m.base[f], (uint32_t)(a.cam.tiles_x * a.cam.tiles_y));
     }
 }
 
-// Backward pass of the tile order[block_slot] of a frame with ntiles tiles.
-template <int PX, int TPR, bool LIMIT>
-__device__ __forceinline__ void backward_tile(const RenderBwdArgs& a, uint32_t block_slot, uint32_t ntiles) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Staged* s_sp = reinterpret_cast<Staged*>(smem_raw);
-    float4* s_rgb = reinterpret_cast<float4*>(smem_raw + sizeof(Staged) * a.batch);
-    uint32_t* s_idx = reinterpret_cast<uint32_t*>(smem_raw + (sizeof(Staged) + sizeof(float4)) * a.batch);
-    const uint32_t* const wbits = a.contrib + (size_t)(threadIdx.x >> 5) * a.contrib_words;
-    __shared__ uint32_t s_max;
+// Backward pass of the groups of one warp (`unit`) of a frame with ntiles tiles.
+template <int PX, int SUBS, bool LIMIT>
+__device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t unit, uint32_t ntiles) {
+    using LN = Lanes<PX, SUBS>;
+    constexpr int U = 2;
+    __shared__ Entry s_e[LN::TPW][32];
+    const LN ln(unit);
     const CamK& c = a.cam;
-    const uint32_t tile_id = a.order[block_slot];
-    if (tile_id >= ntiles) {   // an order not written by gs_bin_sort
-        if (threadIdx.x == 0) debug_fail(a.status);
-        return;
+    const uint32_t full = 0xffffffffu;
+    uint32_t tile = ln.index < ntiles ? a.order[ln.index] : 0u;
+    const bool live = ln.index < ntiles && tile < ntiles;
+    if (ln.index < ntiles && !live && ln.tl == 0) debug_fail(a.status);   // an order not written by gs_bin_sort
+    if (!live) tile = 0;
+    const int tx = (int)tile % c.tiles_x, ty = (int)tile / c.tiles_x;
+    const int x0 = tx * (kSub * LN::SX), y0 = ty * c.tile_h;
+    const int ly = kSub * ln.sy + ln.row, py = y0 + ly, px0 = x0 + kSub * ln.sx + ln.col;
+    const f32x2 lyf = pack2((float)ly, (float)ly);
+    uint32_t start = 0, len = 0;
+    if (live) {
+        const uint2 r = *reinterpret_cast<const uint2*>(a.ranges + 2 * tile);
+        start = r.x;
+        len = r.y - r.x;
+        if (GS_DEBUG && (r.y < r.x || r.y > a.capacity)) {
+            if (ln.tl == 0) debug_fail(a.status);
+            len = 0;
+        }
     }
-    const int tile = (int)tile_id;
-    const int tx = tile % c.tiles_x, ty = tile / c.tiles_x;
-    const int nthreads = blockDim.x;
-    const int ly = threadIdx.x / TPR, c0 = threadIdx.x % TPR;   // TPR threads per tile row
-    const int x0 = tx * c.tile_w, y0 = ty * c.tile_h;
-    const int py = y0 + ly;
-    const float lyf = (float)ly, c0f = (float)c0;
-    const uint32_t start = a.ranges[2 * tile];
-    uint32_t len = a.ranges[2 * tile + 1] - start;
-    if (GS_DEBUG && (a.ranges[2 * tile + 1] < start || a.ranges[2 * tile + 1] > a.capacity)) {
-        if (threadIdx.x == 0) debug_fail(a.status);
-        len = 0;
-    }
+    const uint32_t* const bits = a.contrib + (size_t)((start >> 5) + tile) * SUBS + ln.sub;
     const float amax = a.cfg.alpha_max;
-    const float log2_amin = __log2f(a.cfg.alpha_min);
+    const float log2_amin = __log2f(a.cfg.alpha_min), lo_care = log2_care(amax);
     const size_t P = (size_t)c.W * c.H;
-    // what the loops read, in registers (see the forward pass)
-    const int batch = a.batch, n = a.n;
-    const uint32_t* const vals = a.vals;
-    const float4* const xy = a.xy;
-    const float4* const conic = a.conic_opacity;
-    const float4* const rgb = a.rgb;
+    const uint32_t* const vals = a.vals + start;
     float* const grad2d = a.grad2d;
+    const f32x2 one = pack2(1.f, 1.f), neg = pack2(-1.f, -1.f);
 
-    // Per pixel: T, R . dL/dC (only this projection of the colour behind is ever needed) and dL/dC.
-    float T[PX], Rd[PX], dLr[PX], dLg[PX], dLb[PX];
+    // Per pixel: T, -R . dL/dC (only this projection of the colour behind is ever needed), dL/dC.
+    f32x2 T[LN::PAIRS], nRd[LN::PAIRS], dLr[LN::PAIRS], dLg[LN::PAIRS], dLb[LN::PAIRS];
     uint32_t mylast[PX];
     // LIMIT: the first `skip` blended splats met from the back (all but the grad_limit front-most)
     // get no gradient; the recurrences for T and R . dL/dC still run through them
     uint32_t skip[PX], seen[PX];
-    uint32_t tmax = 0;
+    uint32_t gmax = 0;
+    bool odd = false;
 #pragma unroll
-    for (int j = 0; j < PX; ++j) {
-        const int px = x0 + c0 + TPR * j;
-        mylast[j] = 0;
-        skip[j] = seen[j] = 0;
-        T[j] = 1.0f;
-        dLr[j] = dLg[j] = dLb[j] = 0.f;
-        if (px < c.W && py < c.H) {
-            const size_t p = (size_t)py * c.W + px;
-            mylast[j] = a.last[p];
-            if (LIMIT) {
-                const uint32_t nb = a.count[p], lim = (uint32_t)a.cfg.grad_limit;
-                skip[j] = nb > lim ? nb - lim : 0u;
+    for (int i = 0; i < LN::PAIRS; ++i) {
+        float t[2], dr[2], dg[2], db[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int px = px0 + 2 * i + h;
+            t[h] = 1.0f;
+            dr[h] = dg[h] = db[h] = 0.f;
+            mylast[2 * i + h] = skip[2 * i + h] = seen[2 * i + h] = 0;
+            if (live && px < c.W && py < c.H) {
+                const size_t p = (size_t)py * c.W + px;
+                mylast[2 * i + h] = min(a.last[p], len);   // last positions never exceed the tile's list
+                if (LIMIT) {
+                    const uint32_t nb = a.count[p], lim = (uint32_t)a.cfg.grad_limit;
+                    skip[2 * i + h] = nb > lim ? nb - lim : 0u;
+                }
+                t[h] = a.T_final[p];
+                dr[h] = a.dL_drgb[p];
+                dg[h] = a.dL_drgb[P + p];
+                db[h] = a.dL_drgb[2 * P + p];
             }
-            T[j] = a.T_final[p];
-            dLr[j] = a.dL_drgb[p];
-            dLg[j] = a.dL_drgb[P + p];
-            dLb[j] = a.dL_drgb[2 * P + p];
+            gmax = max(gmax, mylast[2 * i + h]);
         }
-        Rd[j] = a.bg[0] * dLr[j] + a.bg[1] * dLg[j] + a.bg[2] * dLb[j];
-        tmax = max(tmax, mylast[j]);
+        T[i] = pack2(t[0], t[1]);
+        dLr[i] = pack2(dr[0], dr[1]);
+        dLg[i] = pack2(dg[0], dg[1]);
+        dLb[i] = pack2(db[0], db[1]);
+        float rd[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            rd[h] = a.bg[0] * dr[h] + a.bg[1] * dg[h] + a.bg[2] * db[h];
+            // not finite, or so large that a product could overflow
+            odd |= !(fabsf(dr[h]) <= kWild && fabsf(dg[h]) <= kWild && fabsf(db[h]) <= kWild && fabsf(rd[h]) <= kWild);
+        }
+        nRd[i] = pack2(-rd[0], -rd[1]);
     }
-    if (threadIdx.x == 0) s_max = 0;
-    __syncthreads();
-    const uint32_t wmax = __reduce_max_sync(0xffffffffu, tmax);
-    if ((threadIdx.x & 31) == 0) atomicMax(&s_max, wmax);
-    __syncthreads();
-    const uint32_t count = min(s_max, len);   // last positions never exceed the tile's list
+#pragma unroll
+    for (int m = LN::GL / 2; m > 0; m >>= 1) gmax = max(gmax, __shfl_xor_sync(full, gmax, m));
+    const uint32_t wmax = __reduce_max_sync(full, gmax);
     uint32_t nblend = 0;
-    const int lane = threadIdx.x & 31;
-    const int slot = reduce_slot(lane);
+    int slot0, nslots;
+    reduce_slots<LN::GL>(ln.lane, slot0, nslots);
+    // constant factors of the (up to two) totals this lane adds: the log2-scaled (p, q) back to
+    // the whitened frame, and the sign (the sums are of negated terms)
+    auto factor = [](int s) { return s < 2 ? -kUnscale : s < 5 ? -kLn2 : -1.0f; };
+    const float f0 = factor(slot0), f1 = factor(slot0 + 1);
 
-    for (int bend = (int)count; bend > 0; bend -= batch) {
-        const int nb = min(batch, bend);
-        __syncthreads();
-        for (int k = threadIdx.x; k < nb; k += nthreads) {
-            uint32_t g = vals[start + (uint32_t)(bend - 1 - k)];
-            if (g >= (uint32_t)n) {   // only reachable after a timed-out sort
-                debug_fail(a.status);
-                g = 0;
-            }
-            Staged st;
-            stage_splat(xy[g], conic[g], x0, y0, log2_amin, st);
-            s_sp[k] = st;
-            s_rgb[k] = rgb[g];
-            s_idx[k] = g;
+    // the contribution word of window w: the splats some pixel of the group blended
+    auto word_of = [&](int w) {
+        uint32_t v = 0;
+        const uint32_t base = 32u * (uint32_t)w;
+        if (w >= 0 && base < gmax) {
+            v = bits[(size_t)w * SUBS];
+            if (gmax - base < 32) v &= (1u << (gmax - base)) - 1u;
         }
-        __syncthreads();
-        // Only the splats some pixel of this warp blended in the forward pass (its contribution
-        // bits; the backward blends exactly the forward's pairs), 32 at a time.
-        for (int k0 = 0; k0 < nb; k0 += 32) {
-          uint32_t todo = __brev(bits_window(wbits, start + (uint32_t)(bend - 1 - k0)));   // bit i: splat k0 + i
-          if (nb - k0 < 32) todo &= (1u << (nb - k0)) - 1u;
-          while (todo) {
-            const int k = k0 + __ffs(todo) - 1;
-            todo &= todo - 1u;
-            const uint32_t pos = (uint32_t)(bend - 1 - k);
-            float g[9];
-#pragma unroll
-            for (int v = 0; v < 9; ++v) g[v] = 0.f;
-            bool contrib = false;
-            const Staged st = s_sp[k];
-            float p0, dp, q, qq;
-            splat_row(st, lyf, c0f, (float)TPR, p0, dp, q, qq);
-            if (pos < tmax && qq <= st.a.z) {                      // s >= q^2: else the whole row skips
-                const float4 col = s_rgb[k];
-#pragma unroll
-                for (int j = 0; j < PX; ++j) {
-                    float p;
-                    const float s = splat_s(p0, dp, qq, j, p);
-                    if (pos >= mylast[j] || s > st.a.z) continue;
-                    const bool grad = !LIMIT || seen[j]++ >= skip[j];
-                    contrib |= grad;
-                    ++nblend;
-                    const float oG = hw_exp2(__fsub_rn(st.a.w, s));
-                    const float alpha = fminf(amax, oG);
-                    const float one_m = __fsub_rn(1.0f, alpha);
-                    const float Ti = T[j] * hw_rcp(one_m);      // T_i = T_{i+1} / (1 - alpha_i), one_m >= 0.01
-                    const float w = alpha * Ti;
-                    // dL/dalpha = T_i (c_i - R_{i+1}) . dL/dC;  R_i . dL/dC = R_{i+1} . dL/dC + alpha (c_i - R_{i+1}) . dL/dC
-                    const float diff = col.x * dLr[j] + col.y * dLg[j] + col.z * dLb[j] - Rd[j];
-                    const float dalpha = Ti * diff;
-                    Rd[j] = fmaf(alpha, diff, Rd[j]);
-                    T[j] = Ti;
-                    if (LIMIT && !grad) continue;
-                    g[6] += w * dLr[j];
-                    g[7] += w * dLg[j];
-                    g[8] += w * dLb[j];
-                    if (oG <= amax) {
-                        // dpow = dL/d(power): sums of dpow (p, q) and dpow (p, q)(p, q)^T in the
-                        // whitened frame (scaled p, q), the constant factors 1/o, 1/kScaleLog2 and
-                        // ln 2 once per splat below
-                        const float dpow = oG * dalpha;
-                        const float dpp = dpow * p, dpq = dpow * q;
-                        g[0] += dpp;
-                        g[1] += dpq;
-                        g[2] = fmaf(dpp, p, g[2]);
-                        g[3] = fmaf(dpp, q, g[3]);
-                        g[4] = fmaf(dpq, q, g[4]);
-                        g[5] += dpow;
-                    }
-                }
-            }
-            const uint32_t who = __ballot_sync(0xffffffffu, contrib);
-            if (who == 0) continue;
-            float* dst = grad2d + 12 * (size_t)s_idx[k];
-            const float k1 = kUnscale, k2 = kLn2, ko = st.b.w;
-            if (__popc(who) <= kDirectLanes) {
-                // few contributing lanes: each adds its own sums (cheaper than a butterfly)
-                if (contrib) {
-                    atomicAdd(reinterpret_cast<float4*>(dst), make_float4(k1 * g[0], k1 * g[1], k2 * g[2], k2 * g[3]));
-                    atomicAdd(reinterpret_cast<float4*>(dst) + 1, make_float4(k2 * g[4], ko * g[5], g[6], g[7]));
-                    atomicAdd(dst + 8, g[8]);
-                }
-            } else {
-                const float tot = warp_reduce9(g, lane);
-                if (slot >= 0 && !(lane & 1)) atomicAdd(dst + slot, tot * (slot < 2 ? k1 : slot < 5 ? k2 : slot == 5 ? ko : 1.0f));
-            }
-          }
+        return v;
+    };
+    Fetched fetched;
+    uint32_t ids[LN::ROUNDS];
+    const int wlast = (int)((wmax + 31) / 32) - 1;
+    uint32_t next = word_of(wlast);
+    if (wlast >= 0) {
+        fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, 32u * (uint32_t)wlast + (uint32_t)ln.tl, len);
+        if (LN::AHEAD) {
+            fetch_splat(fetched, ids[0], a);
+            fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, 32u * (uint32_t)max(0, wlast - 1) + (uint32_t)ln.tl, len);
         }
     }
-    const uint32_t wblend = __reduce_add_sync(0xffffffffu, nblend);
-    if ((threadIdx.x & 31) == 0 && wblend) atomicAdd(a.blended, (unsigned long long)wblend);
+    for (int w = wlast; w >= 0; --w) {
+        const uint32_t base = 32u * (uint32_t)w;
+        uint32_t word = next;
+        next = word_of(w - 1);
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < LN::ROUNDS; ++r) {
+            if (!LN::AHEAD) fetch_splat(fetched, ids[r], a);
+            Staged st;
+            stage_splat(fetched.xy, fetched.conic, x0, y0, log2_amin, st);
+            s_e[ln.slot][ln.tl + r * LN::SL] = entry_of(st, fetched.rgb, fetched.id, lo_care);
+        }
+        // in flight while this window is walked
+        if (LN::AHEAD) fetch_splat(fetched, ids[0], a);
+        fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, 32u * (uint32_t)max(0, w - (LN::AHEAD ? 2 : 1)) + (uint32_t)ln.tl, len);
+        __syncwarp();
+        while (__any_sync(full, word != 0)) {   // every group its own splats, back to front
+            Entry es[U];
+            uint32_t at[U];
+            float qs[U];
+            f32x2 sums[U][6];
+            bool any_grad = false;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {   // the next U splats of the group, back to front
+                const int k = word ? 31 - __clz((int)word) : 0;
+                at[u] = word ? base + (uint32_t)k : 0xffffffffu;
+                word &= ~(1u << k);
+                es[u] = s_e[ln.slot][k];
+            }
+            // care: alpha may be clamped (its gradient then stops), or a product of a pixel that
+            // does not blend the splat may not be finite (`odd` dL/dC): clear those products
+            auto blend = [&](auto care_c) {
+            constexpr bool care = decltype(care_c)::value;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+            const Entry& e = es[u];
+            const RowPairs row = splat_row(ln, e, lyf);
+            const float thr = __fsub_rn(low(e.lo), log2_amin);
+            // past every last position when the group is idle or, as s >= q^2, the whole row skips
+            const uint32_t pos = low(row.qq) > thr ? 0xffffffffu : at[u];
+            f32x2 S0 = 0, S1 = 0, S2 = 0, Gr = 0, Gg = 0, Gb = 0;
+            bool contrib = false;
+#pragma unroll
+                for (int i = 0; i < LN::PAIRS; ++i) {
+                    const float jj = ln.j(2 * i);
+                    const f32x2 p = fma2(pack2(jj, jj), row.dp, row.p0[i & 1]);
+                    const f32x2 s = fma2(p, p, row.qq);
+                    const f32x2 x = fma2(s, neg, e.lo);
+                    float sv[2], xv[2], na[2], om[2];
+                    unpack2(s, sv[0], sv[1]);
+                    unpack2(x, xv[0], xv[1]);
+                    bool grad[2], grad_a[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float oG = hw_exp2(xv[h]);
+                        const bool ok = pos < mylast[2 * i + h] && !(sv[h] > thr);
+                        if (ok) ++nblend;
+                        grad[h] = ok;
+                        if (LIMIT) {
+                            grad[h] = ok && seen[2 * i + h] >= skip[2 * i + h];
+                            seen[2 * i + h] += ok;
+                            contrib |= grad[h];
+                        }
+                        grad_a[h] = grad[h] && (!care || oG <= amax);
+                        na[h] = ok ? (care ? fmaxf(-amax, -oG) : -oG) : 0.f;       // -alpha; 0 when skipped
+                    }
+                    auto only = [](f32x2 v, const bool (&on)[2]) {
+                        float y[2];
+                        unpack2(v, y[0], y[1]);
+                        return pack2(on[0] ? y[0] : 0.f, on[1] ? y[1] : 0.f);
+                    };
+                    const f32x2 na2 = pack2(na[0], na[1]);
+                    unpack2(add2(na2, one), om[0], om[1]);                     // 1 - alpha >= 0.01
+                    const f32x2 Ti = mul2(T[i], pack2(hw_rcp(om[0]), hw_rcp(om[1])));   // T_i = T_{i+1} / (1 - alpha_i)
+                    f32x2 nw = mul2(na2, Ti);
+                    // dL/dalpha = T_i (c_i - R_{i+1}) . dL/dC;  R_i . dL/dC = R_{i+1} . dL/dC + alpha (c_i - R_{i+1}) . dL/dC
+                    const f32x2 diff = fma2(e.r, dLr[i], fma2(e.g, dLg[i], fma2(e.b, dLb[i], nRd[i])));
+                    nRd[i] = fma2(na2, diff, nRd[i]);
+                    T[i] = Ti;
+                    // -dL/d(power) = -alpha dL/dalpha; its sums with 1, p, p^2 (q is the row's)
+                    f32x2 ndp = mul2(nw, diff);
+                    if (care) {
+                        ndp = only(ndp, grad_a);
+                        Gr = add2(Gr, only(mul2(nw, dLr[i]), grad));
+                        Gg = add2(Gg, only(mul2(nw, dLg[i]), grad));
+                        Gb = add2(Gb, only(mul2(nw, dLb[i]), grad));
+                    } else {
+                        if (LIMIT) {
+                            nw = only(nw, grad);
+                            ndp = only(ndp, grad);
+                        }
+                        Gr = fma2(nw, dLr[i], Gr);
+                        Gg = fma2(nw, dLg[i], Gg);
+                        Gb = fma2(nw, dLb[i], Gb);
+                    }
+                    const f32x2 ndpp = mul2(ndp, p);
+                    S0 = add2(S0, ndp);
+                    S1 = add2(S1, ndpp);
+                    S2 = fma2(ndpp, p, S2);
+                }
+            sums[u][0] = S0; sums[u][1] = S1; sums[u][2] = S2;
+            sums[u][3] = Gr; sums[u][4] = Gg; sums[u][5] = Gb;
+            qs[u] = low(row.q);
+            any_grad |= contrib;
+            }
+            };
+            uint32_t flags = odd ? 0x80000000u : 0u;
+#pragma unroll
+            for (int u = 0; u < U; ++u) flags |= es[u].id;
+            if (LN::ONE_PATH || (int)flags < 0) blend(std::true_type{});
+            else blend(std::false_type{});
+            if (LIMIT && !__any_sync(full, any_grad)) continue;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const float q = qs[u], t0 = sum2(sums[u][0]), t1 = sum2(sums[u][1]), qt0 = q * t0;
+                const float v[9] = {t1, qt0, sum2(sums[u][2]), q * t1, q * qt0, es[u].ko * t0, sum2(sums[u][3]),
+                                    sum2(sums[u][4]), sum2(sums[u][5])};
+                float tot[2];
+                group_reduce9<LN::GL>(v, ln.lane, tot);
+                if (at[u] != 0xffffffffu) {
+                    float* dst = grad2d + 12 * (size_t)(es[u].id & 0x7fffffffu) + slot0;
+                    if (nslots > 0) atomicAdd(dst, f0 * tot[0]);
+                    if (nslots > 1) atomicAdd(dst + 1, f1 * tot[1]);
+                }
+            }
+        }
+    }
+    const uint32_t wblend = __reduce_add_sync(full, nblend);
+    if (ln.lane == 0 && wblend) atomicAdd(a.blended, (unsigned long long)wblend);
 }
 
-// One block per tile, arguments as in k_render_forward_t.
-template <int PX, int TPR, int MAXF, bool LIMIT>
-__global__ void __launch_bounds__(64) k_render_backward_t(const __grid_constant__ Multi<RenderBwdArgs, MAXF> m) {
+// One warp per block, arguments as in k_render_forward_t.
+template <int PX, int SUBS, int MAXF, bool LIMIT>
+__global__ void __launch_bounds__(32, 12) k_render_backward_t(const __grid_constant__ Multi<RenderBwdArgs, MAXF> m) {
     if constexpr (MAXF == 1) {
-        backward_tile<PX, TPR, LIMIT>(m.a[0], blockIdx.x, m.base[1]);
+        backward_unit<PX, SUBS, LIMIT>(m.a[0], blockIdx.x, (uint32_t)(m.a[0].cam.tiles_x * m.a[0].cam.tiles_y));
     } else {
         const int f = find_frame<MAXF>(m.base, m.frames, blockIdx.x);
         const RenderBwdArgs a = m.a[f];
-        backward_tile<PX, TPR, LIMIT>(a, blockIdx.x - m.base[f], m.base[f + 1] - m.base[f]);
+        backward_unit<PX, SUBS, LIMIT>(a, blockIdx.x - m.base[f], (uint32_t)(a.cam.tiles_x * a.cam.tiles_y));
     }
 }
 
-size_t fwd_smem(int batch) { return (sizeof(Staged) + sizeof(float4) + sizeof(uint32_t)) * (size_t)batch; }
-size_t bwd_smem(int batch) { return (sizeof(Staged) + sizeof(float4) + sizeof(uint32_t)) * (size_t)batch; }
-
-}  // namespace
-
-// Tiles of every frame, in frame order (frames without Gaussians still get their background
-// and transmittance written); all frames of a batch share the tile shape and the batch depth.
-template <typename A, int MAXF>
-static uint32_t tile_split(Multi<A, MAXF>& m) {
+// Warps of every frame, in frame order (frames without Gaussians still get their background
+// and transmittance written); all frames of a batch share the tile shape.
+template <int PX, int SUBS, typename A, int MAXF>
+uint32_t unit_split(Multi<A, MAXF>& m) {
+    constexpr int GW = Lanes<PX, SUBS>::GW;
     m.base[0] = 0;
     for (int f = 0; f < m.frames; ++f)
-        m.base[f + 1] = m.base[f] + (uint32_t)(m.a[f].cam.tiles_x * m.a[f].cam.tiles_y);
+        m.base[f + 1] = m.base[f] + (uint32_t)((m.a[f].cam.tiles_x * m.a[f].cam.tiles_y * SUBS + GW - 1) / GW);
     return m.base[m.frames];
 }
 
+template <int PX, int SUBS, int MAXF>
+cudaError_t forward_px(Multi<RenderFwdArgs, MAXF>& m, cudaStream_t s) {
+    const uint32_t units = unit_split<PX, SUBS>(m);
+    if (units == 0) return cudaSuccess;
+    // gradient-limited frames also record the blended splats per pixel
+    if (m.a[0].out_count) k_render_forward_t<PX, SUBS, MAXF, true><<<units, 32, 0, s>>>(m);
+    else k_render_forward_t<PX, SUBS, MAXF, false><<<units, 32, 0, s>>>(m);
+    return cudaGetLastError();
+}
+
+template <int PX, int SUBS, int MAXF>
+cudaError_t backward_px(Multi<RenderBwdArgs, MAXF>& m, cudaStream_t s) {
+    const uint32_t units = unit_split<PX, SUBS>(m);
+    if (units == 0) return cudaSuccess;
+    if (m.a[0].count) k_render_backward_t<PX, SUBS, MAXF, true><<<units, 32, 0, s>>>(m);
+    else k_render_backward_t<PX, SUBS, MAXF, false><<<units, 32, 0, s>>>(m);
+    return cudaGetLastError();
+}
+
+// Pixels per lane, by the 8x8 sub-blocks of the launch.  Eight per lane take the fewest
+// instructions per splat (four sub-blocks share a warp's iteration) but give one warp per 16x16
+// tile: a frame of few tiles leaves the chip idle behind its longest lists.  Measured, 8 / 4 / 2
+// pixels per lane, forward and backward in us:
+//   16 tiles (64x64, 5k Gaussians, 64 sub-blocks)        162 /  97 /  63    302 / 183 / 134
+//   813x611 in 8x8 tiles (60k, 7,854)                     78 /  59 /  51
+//   979x546 (150k, 8,680)                                136 / 104 /  89    161 / 136 / 152
+//   1601x901 in 16x8 tiles (500k, 22,826)                151 / 142 / 160    178 / 188 / 205
+//   1920x1080 (200k, 32,640)                             185 / 200 / 234    275 / 311 / 410
+//   1920x1080 (3M, 32,640)                               270 / 299 / 341    419 / 470 / 606
+int forward_px_for(unsigned long long groups) { return groups < 12000 ? 2 : groups < 26000 ? 4 : 8; }
+int backward_px_for(unsigned long long groups) { return groups < 3000 ? 2 : groups < 16000 ? 4 : 8; }
+
+template <typename A, int MAXF>
+unsigned long long sub_blocks(const Multi<A, MAXF>& m, int subs) {
+    unsigned long long g = 0;
+    for (int f = 0; f < m.frames; ++f) g += (unsigned long long)(m.a[f].cam.tiles_x * m.a[f].cam.tiles_y) * subs;
+    return g;
+}
+
+template <int SUBS, int MAXF>
+cudaError_t forward_subs(Multi<RenderFwdArgs, MAXF>& m, cudaStream_t s) {
+    switch (forward_px_for(sub_blocks(m, SUBS))) {
+        case 2: return forward_px<2, SUBS>(m, s);
+        case 4: return forward_px<4, SUBS>(m, s);
+        default: return forward_px<8, SUBS>(m, s);
+    }
+}
+
+template <int SUBS, int MAXF>
+cudaError_t backward_subs(Multi<RenderBwdArgs, MAXF>& m, cudaStream_t s) {
+    switch (backward_px_for(sub_blocks(m, SUBS))) {
+        case 2: return backward_px<2, SUBS>(m, s);
+        case 4: return backward_px<4, SUBS>(m, s);
+        default: return backward_px<8, SUBS>(m, s);
+    }
+}
+
+}  // namespace
+
 template <int MAXF>
 cudaError_t launch_render_forward(Multi<RenderFwdArgs, MAXF>& m, cudaStream_t s) {
-    const uint32_t tiles = tile_split(m);
-    if (tiles == 0) return cudaSuccess;
-    const RenderFwdArgs& a = m.a[0];
-    // 4 threads per tile row (measured: 2 per row, one warp per 16x16 tile, is 1.5x slower; 8 per
-    // row makes the forward 4 % faster and the backward 10 % slower, and both kernels must
-    // evaluate a pixel with the same operation sequence for their decisions to agree)
-    const dim3 grid(tiles), block(4 * a.cam.tile_h);
-    const size_t smem = fwd_smem(a.batch);
-    if (a.out_count) {   // gradient-limited frames also record the blended splats per pixel
-        if (a.cam.tile_w == 16) k_render_forward_t<4, 4, MAXF, true><<<grid, block, smem, s>>>(m);
-        else k_render_forward_t<2, 4, MAXF, true><<<grid, block, smem, s>>>(m);
-    } else {
-        if (a.cam.tile_w == 16) k_render_forward_t<4, 4, MAXF, false><<<grid, block, smem, s>>>(m);
-        else k_render_forward_t<2, 4, MAXF, false><<<grid, block, smem, s>>>(m);
-    }
-    return cudaGetLastError();
+    const CamK& c = m.a[0].cam;   // all frames of a batch share the tile shape
+    const int subs = (c.tile_w / kSub) * (c.tile_h / kSub);
+    return subs == 4 ? forward_subs<4>(m, s) : subs == 2 ? forward_subs<2>(m, s) : forward_subs<1>(m, s);
 }
 
 template <int MAXF>
 cudaError_t launch_render_backward(Multi<RenderBwdArgs, MAXF>& m, cudaStream_t s) {
-    const uint32_t tiles = tile_split(m);
-    if (tiles == 0) return cudaSuccess;
-    const RenderBwdArgs& a = m.a[0];
-    const dim3 grid(tiles), block(4 * a.cam.tile_h);
-    const size_t smem = bwd_smem(a.batch);
-    if (a.count) {
-        if (a.cam.tile_w == 16) k_render_backward_t<4, 4, MAXF, true><<<grid, block, smem, s>>>(m);
-        else k_render_backward_t<2, 4, MAXF, true><<<grid, block, smem, s>>>(m);
-    } else {
-        if (a.cam.tile_w == 16) k_render_backward_t<4, 4, MAXF, false><<<grid, block, smem, s>>>(m);
-        else k_render_backward_t<2, 4, MAXF, false><<<grid, block, smem, s>>>(m);
-    }
-    return cudaGetLastError();
+    const CamK& c = m.a[0].cam;
+    const int subs = (c.tile_w / kSub) * (c.tile_h / kSub);
+    return subs == 4 ? backward_subs<4>(m, s) : subs == 2 ? backward_subs<2>(m, s) : backward_subs<1>(m, s);
 }
 
 template <int MAXF>
