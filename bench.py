@@ -201,8 +201,14 @@ def row_sort(layout) -> bool:
     return bool(layout.depth_passes) and layout.tiles_x <= 255
 
 
+def fused_launches(layout) -> int:
+    """Passes of launches_per_step that share another's launch: with the row sort, the segment pass
+    zeroes the look-back rows (sort-prepare) and the tile scan writes the tile order."""
+    return 2 if row_sort(layout) else 0
+
+
 def launches_per_step(layout) -> int:
-    """Kernels one step launches: preprocess; binning = two-phase: depth histogram + depth
+    """Passes of one step, one kernel each but for fused_launches: preprocess; binning = two-phase: depth histogram + depth
     passes + one segment pass (count, scan and records), then either sort-prepare + row passes
     over the records + column count + tile scan + column pass (key_passes = row passes + 1) or
     emit + sort-prepare + instance passes + ranges; KEY64: count + pair scan + segment write +
@@ -471,7 +477,7 @@ def run_ours(args, rank, world, local_rank):
         "batch": batch,
         "multi_scene": multi,
         "small_configs": small,
-        "gpu_launches": launches_per_step(fr.layout) * args.steps, "kernels": kernels,
+        "gpu_launches": (launches_per_step(fr.layout) - fused_launches(fr.layout)) * args.steps, "kernels": kernels,
     }
     if rank == 0:
         print(json.dumps(line), flush=True)

@@ -94,6 +94,126 @@ __global__ void __launch_bounds__(256) k_depth_hist(const __grid_constant__ Mult
 }
 
 // ---------------------------------------------------------------------------------------
+// Depth order of a small frame, one block per frame: the four byte passes of the stable radix
+// sort on keys and indices held in shared memory (a warp ranks its contiguous share of the keys,
+// a pass whose byte all keys agree on is skipped), in place of the clear, histogram and four
+// onesweep launches, whose fixed latencies are all there is at these sizes: 1,000 Gaussians 53 ->
+// 15 us of kernels, 5,000 Gaussians 62 -> 30 us (five launches more).  One block is enough up to
+// about 8,192 keys; above, the passes' work outgrows their latency.
+// ---------------------------------------------------------------------------------------
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallItems = kDepthSmallMax / kSmallThreads;
+
+struct DepthSmallShared {
+    uint32_t key[kDepthSmallMax];
+    uint32_t hist[kSmallWarps][256];
+    uint16_t val[kDepthSmallMax];
+    uint32_t scan[33];
+    uint32_t same, visible;
+};
+
+template <int MAXF>
+__global__ void __launch_bounds__(kSmallThreads) k_depth_small(const __grid_constant__ Multi<DepthSmallArgs, MAXF> m) {
+    extern __shared__ __align__(16) unsigned char smem_small[];
+    DepthSmallShared& sh = *reinterpret_cast<DepthSmallShared*>(smem_small);
+    const DepthSmallArgs& a = m.a[blockIdx.x];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t lt = lanemask_lt();
+    for (int r = 0; r < kClearRegions; ++r) {
+        uint32_t* const p = a.clear.ptr[r];
+        for (unsigned long long k = tid; p && k < a.clear.words[r]; k += kSmallThreads) p[k] = 0u;
+    }
+    if (tid == 0) sh.visible = 0;
+    const int n = a.n;
+    // a warp's keys are contiguous: item i of lane l is key w0 + 32 i + l
+    const int items = (n + kSmallThreads - 1) / kSmallThreads;
+    const int w0 = warp * 32 * items;
+    uint32_t key[kSmallItems], val[kSmallItems];
+    uint32_t vis = 0;
+#pragma unroll
+    for (int i = 0; i < kSmallItems; ++i) {
+        const int k = w0 + 32 * i + lane;
+        key[i] = 0xFFFFFFFFu;
+        val[i] = (uint32_t)k;
+        if (i < items && k < n && a.radius[k] > 0) key[i] = __float_as_uint(a.depth[k]);
+        vis += (uint32_t)(key[i] != 0xFFFFFFFFu);
+    }
+    vis = __reduce_add_sync(0xffffffffu, vis);
+    __syncthreads();
+    if (lane == 0 && vis) atomicAdd(&sh.visible, vis);
+    for (int shift = 0; shift < 32; shift += 8) {
+        for (int k = tid; k < kSmallWarps * 256; k += kSmallThreads) (&sh.hist[0][0])[k] = 0;
+        if (tid == 0) sh.same = 0;
+        __syncthreads();
+        uint32_t* const wh = sh.hist[warp];
+        uint32_t pos[kSmallItems];
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i) {
+            if (i >= items) continue;   // block-uniform
+            const bool valid = w0 + 32 * i + lane < n;
+            const uint32_t d = (key[i] >> shift) & 0xFFu;
+            // lanes of the same digit: one ballot per bit, whatever the digits
+            uint32_t peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const uint32_t bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+                peers &= ((d >> b) & 1u) ? bal : ~bal;
+            }
+            const uint32_t below = peers & lt;
+            const uint32_t prev = valid ? wh[d] : 0u;
+            __syncwarp();
+            if (valid && below == 0) wh[d] = prev + (uint32_t)__popc(peers);
+            __syncwarp();
+            pos[i] = prev + (uint32_t)__popc(below);
+        }
+        __syncthreads();
+        uint32_t cnt = 0;
+        uint32_t c[kSmallWarps];   // thread = digit: every warp's count
+        if (tid < 256) {
+#pragma unroll
+            for (int w = 0; w < kSmallWarps; ++w) {
+                c[w] = sh.hist[w][tid];
+                cnt += c[w];
+            }
+            if (cnt == (uint32_t)n) sh.same = 1;
+        }
+        uint32_t total;
+        uint32_t start = block_exclusive_scan<uint32_t>(cnt, sh.scan, &total);
+        if (sh.same) continue;   // block-uniform: this byte orders nothing
+        if (tid < 256) {
+#pragma unroll
+            for (int w = 0; w < kSmallWarps; ++w) {
+                sh.hist[w][tid] = start;
+                start += c[w];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i) {
+            if (i >= items || w0 + 32 * i + lane >= n) continue;
+            const uint32_t p = wh[(key[i] >> shift) & 0xFFu] + pos[i];
+            sh.key[p] = key[i];
+            sh.val[p] = (uint16_t)val[i];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kSmallItems; ++i) {
+            const int k = w0 + 32 * i + lane;
+            if (i >= items || k >= n) continue;
+            key[i] = sh.key[k];
+            val[i] = sh.val[k];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kSmallItems; ++i) {
+        const int k = w0 + 32 * i + lane;
+        if (i < items && k < n) a.order[k] = val[i];
+    }
+    if (tid == 0) *a.num_visible = sh.visible;
+}
+
+// ---------------------------------------------------------------------------------------
 // One LSD digit pass (8 bits at `shift`), stable.
 // ---------------------------------------------------------------------------------------
 template <typename KeyT, int MAXF>
@@ -895,6 +1015,18 @@ __global__ void __launch_bounds__(kDupThreads) k_segments(const __grid_constant_
             }
             __syncthreads();
             const unsigned long long base_s = s_base_s, base_t = s_base_t;
+            // look-back rows of the passes that follow: each is zeroed by the chunk that writes
+            // the first record it covers (the number of records is known only at the end)
+            if (a.row_passes) {
+                const unsigned long long end_s = min(base_s + blk_s, cap);
+                for (unsigned long long r = (base_s + kSortTile - 1) / kSortTile; r * kSortTile < end_s; ++r)
+                    a.row_lb[r * 256 + tid] = 0u;
+                for (unsigned long long r = (base_s + kColChunk - 1) / kColChunk; r * kColChunk < end_s; ++r)
+                    a.col_lb[r * 256 + tid] = 0u;
+                for (unsigned long long r = (base_s + kColChunkMin - 1) / kColChunkMin;
+                     r < kColMinChunks && r * kColChunkMin < end_s; ++r)
+                    a.col_lb[r * 256 + tid] = 0u;
+            }
 
             // segment records: each thread numbers the non-empty rows of its run from the run's
             // exclusive prefix (the runs are in row order, so the records are too)
@@ -1167,22 +1299,17 @@ __global__ void __launch_bounds__(256) k_ranges32(const __grid_constant__ Multi<
     }
 }
 
-// Zero the look-back rows of the first pass of the instance sort, or of the row sort of the
-// segment records (row count depends on a device-side count).
+// Zero the look-back rows of the first pass of the instance sort (the instance count is on the
+// device).
 template <int MAXF>
 __global__ void k_sort_prepare(const __grid_constant__ Multi<SortPrepareArgs, MAXF> m) {
     for (int f = 0; f < m.frames; ++f) {
         const SortPrepareArgs& a = m.a[f];
-        const uint32_t count =
-            min((unsigned long long)(a.count_dev ? *a.count_dev : a.status->num_instances), a.capacity);
+        const uint32_t count = (uint32_t)min((unsigned long long)a.status->num_instances, a.capacity);
         const size_t stride = (size_t)gridDim.x * blockDim.x;
         const uint32_t rows = (count + a.tile_keys - 1) / a.tile_keys;
         const size_t total = (size_t)rows * 256;
         for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < total; k += stride) a.lookback[k] = 0;
-        if (a.lookback2) {
-            const size_t total2 = (size_t)((count + a.tile_keys2 - 1) / a.tile_keys2) * 256;
-            for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < total2; k += stride) a.lookback2[k] = 0;
-        }
     }
 }
 
@@ -1197,6 +1324,15 @@ cudaError_t launch_depth_hist(Multi<DepthHistArgs, MAXF>& m, cudaStream_t s) {
     }
     if (m.base[m.frames] == 0) return cudaSuccess;
     k_depth_hist<MAXF><<<m.base[m.frames], 256, 0, s>>>(m);
+    return cudaGetLastError();
+}
+
+template <int MAXF>
+cudaError_t launch_depth_small(const Multi<DepthSmallArgs, MAXF>& m, cudaStream_t s) {
+    const cudaError_t e = cudaFuncSetAttribute((const void*)k_depth_small<MAXF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sizeof(DepthSmallShared));
+    if (e != cudaSuccess) return e;
+    k_depth_small<MAXF><<<m.frames, kSmallThreads, sizeof(DepthSmallShared), s>>>(m);
     return cudaGetLastError();
 }
 
@@ -1279,6 +1415,7 @@ cudaError_t launch_clear(const Multi<ClearArgs, kMaxFrames>& m, cudaStream_t s) 
 }
 
 #define GS_INSTANTIATE_BINNING(F)                                                                           \
+    template cudaError_t launch_depth_small<F>(const Multi<DepthSmallArgs, F>&, cudaStream_t);                \
     template cudaError_t launch_depth_hist<F>(Multi<DepthHistArgs, F>&, cudaStream_t);                        \
     template cudaError_t launch_onesweep<uint32_t, F>(const Multi<SortPassArgs<uint32_t>, F>&, int, cudaStream_t); \
     template cudaError_t launch_onesweep<unsigned long long, F>(const Multi<SortPassArgs<unsigned long long>, F>&, \

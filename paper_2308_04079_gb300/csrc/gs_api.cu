@@ -106,7 +106,8 @@ bool make_layout(int n, int W, int H, uint64_t cap, const gs_raster_config* cfg,
     L->tile_order = take((size_t)L->tiles * sizeof(uint32_t));
     L->tile_cnt = take((size_t)L->tiles * sizeof(uint32_t));
     // column-count look-back rows, one per chunk of row-sorted segment records
-    L->col_lb_rows = L->row_sort ? (cc + kColChunk - 1) / kColChunk : 0;
+    const size_t rows_big = (cc + kColChunk - 1) / kColChunk, rows_small = (cc + kColChunkMin - 1) / kColChunkMin;
+    L->col_lb_rows = L->row_sort ? std::max(rows_big, std::min(rows_small, (size_t)kColMinChunks)) : 0;
     L->col_lb = L->row_sort ? take(L->col_lb_rows * 256 * sizeof(uint32_t)) : 0;
     L->grad2d = take(nn * 12 * sizeof(float));
     // blended splats per pixel, written by the forward pass when gradients are limited
@@ -401,20 +402,8 @@ gs_status tiles_by_radix(const FrameSet<MAXF>& fs, bool key64, cudaStream_t s) {
 // its column within the row (tilesort.cu).
 template <int MAXF>
 gs_status tiles_by_rows(const FrameSet<MAXF>& fs, cudaStream_t s) {
-    Multi<SortPrepareArgs, MAXF> pm;
-    pm.frames = fs.count;
     int max_passes = 0;
-    for (int v = 0; v < fs.count; ++v) {
-        const Layout& L = fs.L[v];
-        void* ws = fs.f[v]->ws;
-        Control* ctl = control_of(fs, v);
-        pm.a[v] = SortPrepareArgs{at<uint32_t>(ws, L.sort_lb[0]), kSortTile, &ctl->status,
-                                  (unsigned long long)fs.f[v]->capacity, &ctl->counters[30],
-                                  at<uint32_t>(ws, L.col_lb), kColChunk};
-        max_passes = std::max(max_passes, L.row_passes);
-    }
-    if (launch_sort_prepare(pm, s) != cudaSuccess) return GS_ERR_CUDA;
-    phase("sort prepare", s);
+    for (int v = 0; v < fs.count; ++v) max_passes = std::max(max_passes, fs.L[v].row_passes);
     Control* ctl0 = control_of(fs, 0);
     for (int p = 0; p < max_passes; ++p) {
         Multi<SortPassArgs<uint32_t>, MAXF> m;
@@ -463,6 +452,7 @@ gs_status tiles_by_rows(const FrameSet<MAXF>& fs, cudaStream_t s) {
         a.tile_cnt = at<uint32_t>(ws, L.tile_cnt);
         a.lookback = at<uint32_t>(ws, L.col_lb);
         a.ranges = at<uint32_t>(ws, L.ranges);
+        a.order = at<uint32_t>(ws, L.tile_order);
         a.keys_out = at<uint32_t>(ws, L.ikey[(rp + 1) % 2]);   // = keys_sorted_off (key_passes = rp + 1)
         a.vals_out = at<uint32_t>(ws, L.ival[(rp + 1) % 2]);
         a.chunk_counter = &ctl0->counters[16];
@@ -472,7 +462,7 @@ gs_status tiles_by_rows(const FrameSet<MAXF>& fs, cudaStream_t s) {
     if (launch_col_count(c, s) != cudaSuccess) return GS_ERR_CUDA;
     phase("column count", s);
     if (launch_tile_scan(c, s) != cudaSuccess) return GS_ERR_CUDA;
-    phase("tile scan", s);
+    phase("tile scan and order", s);
     for (int v = 0; v < fs.count; ++v) c.a[v].chunk_counter = &ctl0->counters[17];
     const gs_status r = ok(launch_col_scatter(c, s));
     phase("column pass", s);
@@ -500,14 +490,34 @@ gs_status bin_sort_impl(const FrameSet<MAXF>& fs, cudaStream_t s) {
         clr[v].ptr[3] = at<uint32_t>(ws, L.scan_lb);
         clr[v].words[3] = L.scan_lb_rows * 2;
     }
-    gs_status st = clear_regions(fs, clr, s);
-    if (st != GS_OK) return st;
-    phase("clear", s);
+    // frames of at most kDepthSmallMax Gaussians (and few enough tiles for one block to clear):
+    // cleared and depth-sorted by one block each
+    bool small = !key64;
+    for (int v = 0; v < fs.count; ++v)
+        small = small && fs.f[v]->n > 0 && fs.f[v]->n <= kDepthSmallMax && fs.L[v].tiles <= 32768;
+    gs_status st = GS_OK;
+    if (!small) {
+        st = clear_regions(fs, clr, s);
+        if (st != GS_OK) return st;
+        phase("clear", s);
+    }
     Control* ctl0 = control_of(fs, 0);
 
     Multi<ScanArgs, MAXF> d;
     d.frames = fs.count;
-    if (!key64) {
+    if (small) {
+        Multi<DepthSmallArgs, MAXF> q;
+        q.frames = fs.count;
+        for (int v = 0; v < fs.count; ++v) {
+            const Layout& L = fs.L[v];
+            void* ws = fs.f[v]->ws;
+            q.a[v] = DepthSmallArgs{fs.f[v]->n, at<float>(ws, L.depth), at<int>(ws, L.radius),
+                                    at<uint32_t>(ws, L.gval[(kDepthPasses - 1) % 2]), &control_of(fs, v)->counters[31],
+                                    clr[v]};
+        }
+        if (launch_depth_small(q, s) != cudaSuccess) return GS_ERR_CUDA;
+        phase("depth order", s);
+    } else if (!key64) {
         // Phase 1: stable sort of every frame's Gaussians by fp32 depth bits (culled ones last).
         Multi<DepthHistArgs, MAXF> h;
         h.frames = fs.count;
@@ -580,6 +590,8 @@ gs_status bin_sort_impl(const FrameSet<MAXF>& fs, cudaStream_t s) {
             a.row_passes = 0;
         }
         a.num_segments = &ctl->counters[30];
+        a.row_lb = at<uint32_t>(ws, L.sort_lb[0]);
+        a.col_lb = at<uint32_t>(ws, L.col_lb);
         a.capacity = f->capacity;
         a.hist = &ctl->hist_keys[0][0];
         a.pairs = at<unsigned long long>(ws, L.pairs);
@@ -605,14 +617,17 @@ gs_status bin_sort_impl(const FrameSet<MAXF>& fs, cudaStream_t s) {
         st = tiles_by_rows(rows, s);
         if (st != GS_OK) return st;
     }
-    // the render passes' block order: every frame's tiles by decreasing list length
-    Multi<TileOrderArgs, MAXF> o;
-    o.frames = fs.count;
-    for (int v = 0; v < fs.count; ++v)
-        o.a[v] = TileOrderArgs{at<uint32_t>(fs.f[v]->ws, fs.L[v].ranges), at<uint32_t>(fs.f[v]->ws, fs.L[v].tile_order),
-                               fs.L[v].tiles};
-    st = ok(launch_tile_order(o, s));
-    phase("tile order", s);
+    // the render passes' block order: every frame's tiles by decreasing list length (the row sort
+    // writes it with the ranges)
+    if (radix.count) {
+        Multi<TileOrderArgs, MAXF> o;
+        o.frames = radix.count;
+        for (int v = 0; v < radix.count; ++v)
+            o.a[v] = TileOrderArgs{at<uint32_t>(radix.f[v]->ws, radix.L[v].ranges),
+                                   at<uint32_t>(radix.f[v]->ws, radix.L[v].tile_order), radix.L[v].tiles};
+        st = ok(launch_tile_order(o, s));
+        phase("tile order", s);
+    }
     return st;
 }
 

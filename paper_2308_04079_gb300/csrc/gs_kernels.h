@@ -189,6 +189,8 @@ struct ScanArgs {
     int row_passes;            // > 0: row-segmented tile sort (row_key records, no seg_off, digit
                                // histograms of the row's row_passes bytes into hist)
     uint32_t* num_segments;
+    uint32_t* row_lb;          // row_passes > 0: look-back rows of the first row pass and of the
+    uint32_t* col_lb;          // column count, zeroed as the records that need them are written
     unsigned long long capacity;
     uint32_t* hist;            // [4][256] depth-digit histograms (KEY64), row digits (row_passes > 0)
     unsigned long long* lookback;  // [entries / kDupThreads], zeroed
@@ -227,9 +229,18 @@ struct SortPrepareArgs {
     int tile_keys;             // keys per chunk of the pass that follows
     const gs_device_status* status;
     unsigned long long capacity;
-    const uint32_t* count_dev; // keys of that pass; null: the instance count
-    uint32_t* lookback2;       // optional second table (256 words per row), or null
-    int tile_keys2;            // keys per row of the second table
+};
+
+// Depth order of frames of at most kDepthSmallMax Gaussians: one block per frame sorts in shared
+// memory (k_depth_small), which also clears what the binning stage needs zeroed.
+constexpr int kDepthSmallMax = 8192;
+struct DepthSmallArgs {
+    int n;
+    const float* depth;
+    const int* radius;
+    uint32_t* order;           // [n] out: indices by depth, culled ones last
+    uint32_t* num_visible;     // out
+    ClearArgs clear;
 };
 
 // Row-segmented tile sort (TWO_PHASE, tiles_x <= kRowSortMaxCols).  A segment record is one
@@ -242,7 +253,16 @@ struct SortPrepareArgs {
 // the ranges; the column pass expands the records into instances and stable-ranks them by
 // column within their row, writing each to its final slot.
 constexpr int kRowSortMaxCols = 255;
-constexpr int kColChunk = 2048;   // row-sorted records per chunk of the count and column passes
+// Row-sorted records per chunk of the count and column passes: kColChunk, or fewer while the
+// launch has so few records that its chunks would not fill the chip (col_chunk).
+constexpr int kColChunk = 2048;
+constexpr int kColChunkMin = 256;
+constexpr uint32_t kColMinChunks = 1824;   // 12 per SM
+__host__ __device__ constexpr uint32_t col_chunk(unsigned long long records) {
+    uint32_t c = kColChunkMin;
+    while (c < (uint32_t)kColChunk && records > (unsigned long long)c * kColMinChunks) c *= 2;
+    return c;
+}
 constexpr int kRowKeyRowShift = 17;
 __host__ __device__ constexpr uint32_t row_key(uint32_t row, uint32_t len, uint32_t col) {
     return row << kRowKeyRowShift | len << 8 | col;
@@ -258,6 +278,7 @@ struct ColArgs {
     uint32_t* lookback;            // [chunks][256] per column: counts of a chunk's last row
                                    // (inclusive within the row), zeroed before the count pass
     uint32_t* ranges;              // [2 * tiles]
+    uint32_t* order;               // [tiles] render order (k_tile_scan)
     uint32_t* keys_out;            // [K] tile id per instance
     uint32_t* vals_out;            // [K] Gaussian per instance
     uint32_t* chunk_counter;       // zeroed
@@ -319,6 +340,7 @@ struct TileOrderArgs {
 int persistent_grid(const void* kernel, int threads);
 template <int MAXF> cudaError_t launch_preprocess(Multi<PreprocessArgs, MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_preprocess_backward(BwdPlan<MAXF>& m, cudaStream_t s);
+template <int MAXF> cudaError_t launch_depth_small(const Multi<DepthSmallArgs, MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_depth_hist(Multi<DepthHistArgs, MAXF>& m, cudaStream_t s);
 template <typename KeyT, int MAXF>
 cudaError_t launch_onesweep(const Multi<SortPassArgs<KeyT>, MAXF>& m, int max_chunks, cudaStream_t s);

@@ -52,7 +52,7 @@
 // clamp decisions agree bit for bit.
 //
 // Block order: warps take the tiles in the order of order[], the frame's tiles by decreasing list
-// length (k_tile_order, run at the end of the binning stage).  The work of a tile grows with its
+// length (tilesort.cu).  The work of a tile grows with its
 // list and varies by a factor of several across a frame; blocks start roughly in index order, so
 // in row-major order the longest tiles (the frame's centre) could start late and finish alone.
 #include <type_traits>
@@ -324,68 +324,6 @@ __device__ __forceinline__ void reduce_slots(int lane, int& first, int& n) {
             n = n < half ? n : half;
         }
         len = half;
-    }
-}
-
-constexpr int kOrderThreads = 1024;
-constexpr int kOrderWarps = kOrderThreads / 32;
-constexpr int kOrderBuckets = 128;   // = 4 per lane of the scan warp
-
-// Bucket of a tile's list length: four per octave (the leading bit and the two below it),
-// longer lists in higher buckets; lengths below 2^30 reach bucket 120 at most.
-__device__ __forceinline__ int order_bucket(uint32_t len) {
-    if (len == 0) return 0;
-    const int e = 31 - __clz(len);
-    const uint32_t frac = e >= 2 ? (len >> (e - 2)) & 3u : (len << (2 - e)) & 3u;
-    return min(kOrderBuckets - 1, 1 + 4 * e + (int)frac);
-}
-
-// One block per frame: a stable counting sort of the tiles by decreasing bucket.  Warp w takes
-// a contiguous range of tiles: it counts its range per bucket (its own row of s_pos), a scan over
-// buckets (in decreasing order) and warps turns the counts into first positions, and each warp
-// places its range in tile order.
-template <int MAXF>
-__global__ void __launch_bounds__(kOrderThreads) k_tile_order(const __grid_constant__ Multi<TileOrderArgs, MAXF> m) {
-    __shared__ uint32_t s_pos[kOrderWarps][kOrderBuckets];
-    __shared__ uint32_t s_tot[kOrderBuckets];
-    const TileOrderArgs& a = m.a[blockIdx.x];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles = a.tiles;
-    const int per = ((tiles + kOrderThreads - 1) / kOrderThreads) * 32;   // tiles per warp, a multiple of 32
-    const int t_lo = min(tiles, warp * per), t_hi = min(tiles, t_lo + per);
-    for (int b = lane; b < kOrderBuckets; b += 32) s_pos[warp][b] = 0;
-    __syncwarp();
-    for (int t = t_lo + lane; t < t_hi; t += 32) atomicAdd(&s_pos[warp][order_bucket(a.ranges[2 * t + 1] - a.ranges[2 * t])], 1u);
-    __syncthreads();
-    if (threadIdx.x < kOrderBuckets) {
-        uint32_t sum = 0;
-        for (int w = 0; w < kOrderWarps; ++w) sum += s_pos[w][threadIdx.x];
-        s_tot[threadIdx.x] = sum;
-    }
-    __syncthreads();
-    if (warp == 0) {   // lane l: buckets 127 - 4l, ..., 124 - 4l
-        uint32_t c[4], sum = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { c[e] = s_tot[kOrderBuckets - 1 - 4 * lane - e]; sum += c[e]; }
-        uint32_t run = warp_inclusive_scan<uint32_t>(sum) - sum;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { s_tot[kOrderBuckets - 1 - 4 * lane - e] = run; run += c[e]; }
-    }
-    __syncthreads();
-    if (threadIdx.x < kOrderBuckets) {
-        uint32_t run = s_tot[threadIdx.x];
-        for (int w = 0; w < kOrderWarps; ++w) { const uint32_t c = s_pos[w][threadIdx.x]; s_pos[w][threadIdx.x] = run; run += c; }
-    }
-    __syncthreads();
-    for (int t0 = t_lo; t0 < t_hi; t0 += 32) {   // warp-uniform
-        const int t = t0 + lane;
-        const int b = t < t_hi ? order_bucket(a.ranges[2 * t + 1] - a.ranges[2 * t]) : -1;
-        const uint32_t peers = __match_any_sync(0xffffffffu, b);
-        const uint32_t rank = __popc(peers & lanemask_lt());
-        if (b >= 0) a.order[s_pos[warp][b] + rank] = (uint32_t)t;
-        __syncwarp();
-        if (b >= 0 && rank == 0) s_pos[warp][b] += __popc(peers);
-        __syncwarp();
     }
 }
 
@@ -945,14 +883,6 @@ cudaError_t launch_render_backward(Multi<RenderBwdArgs, MAXF>& m, cudaStream_t s
     return subs == 4 ? backward_subs<4>(m, s) : subs == 2 ? backward_subs<2>(m, s) : backward_subs<1>(m, s);
 }
 
-template <int MAXF>
-cudaError_t launch_tile_order(const Multi<TileOrderArgs, MAXF>& m, cudaStream_t s) {
-    k_tile_order<MAXF><<<m.frames, kOrderThreads, 0, s>>>(m);
-    return cudaGetLastError();
-}
-
-template cudaError_t launch_tile_order<1>(const Multi<TileOrderArgs, 1>&, cudaStream_t);
-template cudaError_t launch_tile_order<kMaxFrames>(const Multi<TileOrderArgs, kMaxFrames>&, cudaStream_t);
 template cudaError_t launch_render_forward<1>(Multi<RenderFwdArgs, 1>&, cudaStream_t);
 template cudaError_t launch_render_forward<kMaxFrames>(Multi<RenderFwdArgs, kMaxFrames>&, cudaStream_t);
 template cudaError_t launch_render_backward<1>(Multi<RenderBwdArgs, 1>&, cudaStream_t);
