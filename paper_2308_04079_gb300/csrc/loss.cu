@@ -15,8 +15,15 @@
 // dS/dmx, dS/dExx, dS/dExy (w is symmetric).  Pass 1 computes the moments, S, L1 and the
 // coefficient maps; pass 2 windows the coefficient maps and forms dL/dx.  Both passes are
 // separable 11-tap convolutions on 32x32 output tiles (the three channels in turn), staged with
-// their halo in shared memory; a thread computes consecutive outputs of each 1-D window from
-// registers, reading each input once for all of them.
+// their halo in shared memory.  Bound by the instructions of the windows: a thread computes four
+// consecutive outputs of a row, then eight of a column, from registers, reading each input once for
+// all of them, and the pairs (x, y), (x^2, y^2) and (a, b) go through packed arithmetic.  The window
+// weights come with the arguments: computing them in fp64 in every block cost more than a third of
+// both passes.  1080p: 111 + 92 us with scalar maps, two and four outputs per thread and in-kernel
+// weights (210 us a call), now 131 us a call against 11 us for its 75 MB of images.
+#include <cmath>
+#include <cstring>
+
 #include "gs_device.cuh"
 #include "gs_kernels.h"
 
@@ -26,131 +33,163 @@ namespace {
 constexpr int kWin = 11, kHalf = 5;
 constexpr int kTile = 32;
 constexpr int kIn = kTile + 2 * kHalf;   // 42
-constexpr int kRowsPer = 4;              // output rows per thread in the vertical passes (256 threads)
-constexpr int kColsPer = 2;              // output columns per thread in the horizontal passes
-static_assert(kTile * kTile == 256 * kRowsPer, "one row group per thread");
-
-// Normalised 1-D Gaussian window, sigma 1.5 (the 2-D window is its outer product), computed by
-// every block into shared memory.
-__device__ __forceinline__ void load_window(float* w) {
-    if (threadIdx.x < kWin) {
-        double sum = 0.0;
-        for (int k = 0; k < kWin; ++k) sum += exp(-(double)((k - kHalf) * (k - kHalf)) / (2.0 * 1.5 * 1.5));
-        const int t = (int)threadIdx.x - kHalf;
-        w[threadIdx.x] = (float)(exp(-(double)(t * t) / (2.0 * 1.5 * 1.5)) / sum);
-    }
-}
+constexpr int kLossThreads = 128;
+constexpr int kRowsPer = 8;              // output rows per thread in the vertical passes
+constexpr int kColsPer = 4;              // output columns per thread in the horizontal passes
+static_assert(kTile * kTile == kLossThreads * kRowsPer, "one row group per thread");
+constexpr int kItems = kIn * (kTile / kColsPer);   // (row, column group) items of a horizontal pass
+// Row strides in elements: odd, so that lanes on consecutive rows hit different banks.
+constexpr int kInStride = kIn + 1, kRowStride = kTile + 1;
 
 struct LossArgs {
     const float* img;     // [3, H, W]
     const float* target;  // [3, H, W]
     int W, H;
     float lambda;
-    float* coef;          // [3 channels][3 maps][H * W]: dS/dmx, dS/dExx, dS/dExy
+    float2* coef_ab;      // [3 channels][H * W]: dS/dmx, dS/dExx
+    float* coef_c;        // [3 channels][H * W]: dS/dExy
+    // normalised 1-D Gaussian window, sigma 1.5 (the 2-D one is its outer product), once and in pairs
+    float win[kWin];
+    f32x2 win2[kWin];
     double* partial;      // [blocks][2]: sums of S and |x - y| of every tile
     unsigned int* done;   // block counter of pass 1 (zeroed)
     float* out_loss;      // [3]: L, L1, mean SSIM
     float* dL_dimg;       // [3, H, W]
 };
 
-__device__ __forceinline__ float load0(const float* p, int W, int H, int x, int y) {
-    return (x >= 0 && x < W && y >= 0 && y < H) ? p[(size_t)y * W + x] : 0.f;
-}
+// The part of a tile's staged inputs one thread moves: column `col` of rows row, row + 3, ... (42
+// columns x 3 rows = 126 of the 128 threads).  Pass 1 fetches the next channel's while this one is
+// windowed (load latency was most of its stalls); pass 2 gains more from a sixth block per SM.
+constexpr int kFetch = kIn / 3;
+static_assert(kIn % 3 == 0 && 3 * kIn <= kLossThreads, "three rows per trip");
+struct Fetch {
+    int col, row, y0;
+    bool on;
+    const size_t at;      // of the first row's element in the image (valid where `on` and in range)
+    __device__ __forceinline__ Fetch(const LossArgs& a, int bx, int by)
+        : col(threadIdx.x % kIn), row(threadIdx.x / kIn), y0(by + (int)threadIdx.x / kIn - kHalf),
+          on((int)threadIdx.x < 3 * kIn && bx + col - kHalf >= 0 && bx + col - kHalf < a.W),
+          at((size_t)((long long)y0 * a.W + bx + col - kHalf)) {}
+    __device__ __forceinline__ bool in(const LossArgs& a, int i) const {
+        return on && (unsigned)(y0 + 3 * i) < (unsigned)a.H;
+    }
+    __device__ __forceinline__ size_t of(const LossArgs& a, int i) const { return at + (size_t)(3 * i) * a.W; }
+    __device__ __forceinline__ bool stages() const { return (int)threadIdx.x < 3 * kIn; }
+    __device__ __forceinline__ int slot(int i) const { return (row + 3 * i) * kInStride + col; }
+};
 
 // Pass 1: window moments, SSIM, L1 and the coefficient maps of one 32x32 tile, all channels.
-__global__ void __launch_bounds__(256) k_ssim_forward(LossArgs a) {
-    __shared__ float s_x[kIn][kIn + 1], s_y[kIn][kIn + 1];
-    __shared__ float s_h[5][kIn][kTile + 1];   // horizontally windowed x, y, x^2, y^2, x y
+__global__ void __launch_bounds__(kLossThreads, 5) k_ssim_forward(const __grid_constant__ LossArgs a) {
+    __shared__ float2 s_in[kIn * kInStride];                                   // (x, y)
+    __shared__ float2 s_m[kIn * kRowStride], s_q[kIn * kRowStride];            // windowed (x, y), (x^2, y^2)
+    __shared__ float s_p[kIn * kRowStride];                                    // windowed x y
     __shared__ double s_red[2][8];
-    __shared__ float c_win[kWin];
-    load_window(c_win);
     const int tid = threadIdx.x;
     const int bx = blockIdx.x * kTile, by = blockIdx.y * kTile;
     const size_t P = (size_t)a.W * a.H;
-    __syncthreads();
-    float w[kWin];   // the window in registers
-#pragma unroll
-    for (int t = 0; t < kWin; ++t) w[t] = c_win[t];
-    // per-thread sums of at most 3 x 4 terms in [-1, 1] and [0, 1] stay in fp32; blocks and the
+    // per-thread sums of at most 3 x 8 terms in [-1, 1] and [0, 1] stay in fp32; blocks and the
     // grid sum in fp64
     float sum_s = 0.f, sum_l1 = 0.f;
-    for (int ch = 0; ch < 3; ++ch) {
-    const float* x = a.img + ch * P;
-    const float* y = a.target + ch * P;
-    __syncthreads();   // the previous channel's reads of s_x, s_y and s_h are done
-    for (int k = tid; k < kIn * kIn; k += blockDim.x) {
-        const int r = k / kIn, cc = k % kIn;
-        s_x[r][cc] = load0(x, a.W, a.H, bx + cc - kHalf, by + r - kHalf);
-        s_y[r][cc] = load0(y, a.W, a.H, bx + cc - kHalf, by + r - kHalf);
-    }
-    __syncthreads();
-    // horizontal windows: a thread takes kColsPer consecutive columns of one row, reading the
-    // kColsPer + 10 inputs they need once
-    for (int k = tid; k < kIn * (kTile / kColsPer); k += blockDim.x) {
-        const int r = k / (kTile / kColsPer), c0 = (k % (kTile / kColsPer)) * kColsPer;
-        float h[5][kColsPer];
+    const Fetch f(a, bx, by);
+    float fx[kFetch], fy[kFetch];
+    auto fetch = [&](int ch) {
 #pragma unroll
-        for (int mm = 0; mm < 5; ++mm)
-#pragma unroll
-            for (int j = 0; j < kColsPer; ++j) h[mm][j] = 0.f;
-#pragma unroll
-        for (int cc = 0; cc < kColsPer + kWin - 1; ++cc) {
-            const float xv = s_x[r][c0 + cc], yv = s_y[r][c0 + cc];
-            const float xx = xv * xv, yy = yv * yv, xy = xv * yv;
-#pragma unroll
-            for (int j = 0; j < kColsPer; ++j)
-                if (cc - j >= 0 && cc - j < kWin) {
-                    const float wt = w[cc - j];
-                    h[0][j] += wt * xv;
-                    h[1][j] += wt * yv;
-                    h[2][j] += wt * xx;
-                    h[3][j] += wt * yy;
-                    h[4][j] += wt * xy;
-                }
+        for (int i = 0; i < kFetch; ++i) {
+            fx[i] = f.in(a, i) ? a.img[ch * P + f.of(a, i)] : 0.f;
+            fy[i] = f.in(a, i) ? a.target[ch * P + f.of(a, i)] : 0.f;
         }
+    };
+    fetch(0);
+    for (int ch = 0; ch < 3; ++ch) {
+        __syncthreads();   // the previous channel's reads of the staged maps are done
+        if (f.stages())
 #pragma unroll
-        for (int mm = 0; mm < 5; ++mm)
+            for (int i = 0; i < kFetch; ++i) s_in[f.slot(i)] = make_float2(fx[i], fy[i]);
+        __syncthreads();
+        // horizontal windows: lanes take consecutive rows of one column group
+        for (int k = tid; k < kItems; k += kLossThreads) {
+            const int c0 = (k / kIn) * kColsPer, r = k % kIn;
+            f32x2 m[kColsPer], q[kColsPer];
+            float p[kColsPer];
 #pragma unroll
-            for (int j = 0; j < kColsPer; ++j) s_h[mm][r][c0 + j] = h[mm][j];
-    }
-    __syncthreads();
-    const float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
-    // vertical windows: a thread takes kRowsPer consecutive rows of one column, reading the
-    // kRowsPer + 10 rows they need once per map
-    {
-        const int cc = tid % kTile, r0 = (tid / kTile) * kRowsPer;
-        float mom[5][kRowsPer];
+            for (int j = 0; j < kColsPer; ++j) {
+                m[j] = q[j] = 0;
+                p[j] = 0.f;
+            }
 #pragma unroll
-        for (int mm = 0; mm < 5; ++mm) {
+            for (int cc = 0; cc < kColsPer + kWin - 1; ++cc) {
+                const float2 v = s_in[r * kInStride + c0 + cc];
+                const f32x2 v2 = pack2(v.x, v.y), vv = mul2(v2, v2);
+                const float xy = v.x * v.y;
 #pragma unroll
-            for (int j = 0; j < kRowsPer; ++j) mom[mm][j] = 0.f;
+                for (int j = 0; j < kColsPer; ++j)
+                    if (cc - j >= 0 && cc - j < kWin) {
+                        const float w = a.win[cc - j];
+                        const f32x2 w2 = a.win2[cc - j];
+                        m[j] = fma2(w2, v2, m[j]);
+                        q[j] = fma2(w2, vv, q[j]);
+                        p[j] = fmaf(w, xy, p[j]);
+                    }
+            }
 #pragma unroll
-            for (int rr = 0; rr < kRowsPer + kWin - 1; ++rr) {
-                const float v = s_h[mm][r0 + rr][cc];
-#pragma unroll
-                for (int j = 0; j < kRowsPer; ++j)
-                    if (rr - j >= 0 && rr - j < kWin) mom[mm][j] += w[rr - j] * v;
+            for (int j = 0; j < kColsPer; ++j) {
+                float2 o;
+                unpack2(m[j], o.x, o.y);
+                s_m[r * kRowStride + c0 + j] = o;
+                unpack2(q[j], o.x, o.y);
+                s_q[r * kRowStride + c0 + j] = o;
+                s_p[r * kRowStride + c0 + j] = p[j];
             }
         }
+        if (ch < 2) fetch(ch + 1);
+        __syncthreads();
+        const float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
+        // vertical windows: a thread takes kRowsPer consecutive rows of one column
+        const int cc = tid % kTile, r0 = (tid / kTile) * kRowsPer;
+        f32x2 mm[kRowsPer], qq[kRowsPer];
+        float pp[kRowsPer];
+#pragma unroll
+        for (int j = 0; j < kRowsPer; ++j) {
+            mm[j] = qq[j] = 0;
+            pp[j] = 0.f;
+        }
+#pragma unroll
+        for (int rr = 0; rr < kRowsPer + kWin - 1; ++rr) {
+            const float2 m = s_m[(r0 + rr) * kRowStride + cc], q = s_q[(r0 + rr) * kRowStride + cc];
+            const float p = s_p[(r0 + rr) * kRowStride + cc];
+            const f32x2 m2 = pack2(m.x, m.y), q2 = pack2(q.x, q.y);
+#pragma unroll
+            for (int j = 0; j < kRowsPer; ++j)
+                if (rr - j >= 0 && rr - j < kWin) {
+                    const float w = a.win[rr - j];
+                    const f32x2 w2 = a.win2[rr - j];
+                    mm[j] = fma2(w2, m2, mm[j]);
+                    qq[j] = fma2(w2, q2, qq[j]);
+                    pp[j] = fmaf(w, p, pp[j]);
+                }
+        }
+        float2* const ab = a.coef_ab + ch * P;
+        float* const cm = a.coef_c + ch * P;
 #pragma unroll
         for (int j = 0; j < kRowsPer; ++j) {
             const int r = r0 + j;
             const int px = bx + cc, py = by + r;
             if (px >= a.W || py >= a.H) continue;
-            const float mx = mom[0][j], my = mom[1][j], exx = mom[2][j], eyy = mom[3][j], exy = mom[4][j];
+            float mx, my, exx, eyy;
+            unpack2(mm[j], mx, my);
+            unpack2(qq[j], exx, eyy);
+            const float exy = pp[j];
             const float A1 = 2.f * mx * my + C1, A2 = 2.f * (exy - mx * my) + C2;
             const float B1 = mx * mx + my * my + C1, B2 = (exx - mx * mx) + (eyy - my * my) + C2;
             const float inv = 1.f / (B1 * B2);
             const float S = A1 * A2 * inv;
-            const size_t q = (size_t)py * a.W + px;
-            float* coef = a.coef + (size_t)ch * 3 * P;
-            coef[q] = 2.f * my * (A2 - A1) * inv - 2.f * mx * S * (B2 - B1) * inv;
-            coef[P + q] = -S / B2;
-            coef[2 * P + q] = 2.f * A1 * inv;
+            const size_t at = (size_t)py * a.W + px;
+            ab[at] = make_float2(2.f * my * (A2 - A1) * inv - 2.f * mx * S * (B2 - B1) * inv, -S / B2);
+            cm[at] = 2.f * A1 * inv;
             sum_s += S;
-            sum_l1 += fabsf(s_x[r + kHalf][cc + kHalf] - s_y[r + kHalf][cc + kHalf]);
+            const float2 v = s_in[(r + kHalf) * kInStride + cc + kHalf];
+            sum_l1 += fabsf(v.x - v.y);
         }
-    }
     }
     // block sums (fixed order), then the last block adds the tiles in index order
     double d_s = sum_s, d_l1 = sum_l1;
@@ -207,79 +246,107 @@ __global__ void __launch_bounds__(256) k_ssim_forward(LossArgs a) {
 }
 
 // Pass 2: dL/dx = (1 - lambda) sign(x - y) / N - lambda / N [(w * a) + 2 x (w * b) + y (w * c)].
-__global__ void __launch_bounds__(256) k_ssim_backward(LossArgs a) {
-    __shared__ float s_c[3][kIn][kIn + 1];
-    __shared__ float s_h[3][kIn][kTile + 1];
-    __shared__ float c_win[kWin];
-    load_window(c_win);
+__global__ void __launch_bounds__(kLossThreads, 6) k_ssim_backward(const __grid_constant__ LossArgs a) {
+    __shared__ float2 s_ab[kIn * kInStride], s_hab[kIn * kRowStride];   // (a, b), staged and windowed by rows
+    __shared__ float s_c[kIn * kInStride], s_hc[kIn * kRowStride];      // c
     const int tid = threadIdx.x;
     const int bx = blockIdx.x * kTile, by = blockIdx.y * kTile;
     const size_t P = (size_t)a.W * a.H;
     const float invN = 1.0f / (3.0f * (float)P);
-    __syncthreads();
-    float w[kWin];   // the window in registers
+    const Fetch f(a, bx, by);
+    float2 fab[kFetch];
+    float fc[kFetch];
+    auto fetch = [&](int ch) {
 #pragma unroll
-    for (int t = 0; t < kWin; ++t) w[t] = c_win[t];
+        for (int i = 0; i < kFetch; ++i) {
+            fab[i] = f.in(a, i) ? a.coef_ab[ch * P + f.of(a, i)] : make_float2(0.f, 0.f);
+            fc[i] = f.in(a, i) ? a.coef_c[ch * P + f.of(a, i)] : 0.f;
+        }
+    };
     for (int ch = 0; ch < 3; ++ch) {
-    const float* coef = a.coef + (size_t)ch * 3 * P;
-    __syncthreads();   // the previous channel's reads of s_c and s_h are done
-    for (int k = tid; k < kIn * kIn; k += blockDim.x) {
-        const int r = k / kIn, cc = k % kIn;
+        fetch(ch);
+        __syncthreads();   // the previous channel's reads of the staged maps are done
+        if (f.stages())
 #pragma unroll
-        for (int mmap = 0; mmap < 3; ++mmap)
-            s_c[mmap][r][cc] = load0(coef + mmap * P, a.W, a.H, bx + cc - kHalf, by + r - kHalf);
-    }
-    __syncthreads();
-    for (int k = tid; k < kIn * (kTile / kColsPer); k += blockDim.x) {
-        const int r = k / (kTile / kColsPer), c0 = (k % (kTile / kColsPer)) * kColsPer;
-        float h[3][kColsPer];
+            for (int i = 0; i < kFetch; ++i) {
+                s_ab[f.slot(i)] = fab[i];
+                s_c[f.slot(i)] = fc[i];
+            }
+        __syncthreads();
+        for (int k = tid; k < kItems; k += kLossThreads) {
+            const int c0 = (k / kIn) * kColsPer, r = k % kIn;
+            f32x2 h[kColsPer];
+            float hc[kColsPer];
 #pragma unroll
-        for (int mm = 0; mm < 3; ++mm)
+            for (int j = 0; j < kColsPer; ++j) {
+                h[j] = 0;
+                hc[j] = 0.f;
+            }
 #pragma unroll
-            for (int j = 0; j < kColsPer; ++j) h[mm][j] = 0.f;
-#pragma unroll
-        for (int cc = 0; cc < kColsPer + kWin - 1; ++cc) {
-#pragma unroll
-            for (int mm = 0; mm < 3; ++mm) {
-                const float v = s_c[mm][r][c0 + cc];
+            for (int cc = 0; cc < kColsPer + kWin - 1; ++cc) {
+                const float2 v = s_ab[r * kInStride + c0 + cc];
+                const float c = s_c[r * kInStride + c0 + cc];
+                const f32x2 v2 = pack2(v.x, v.y);
 #pragma unroll
                 for (int j = 0; j < kColsPer; ++j)
-                    if (cc - j >= 0 && cc - j < kWin) h[mm][j] += w[cc - j] * v;
+                    if (cc - j >= 0 && cc - j < kWin) {
+                        const float w = a.win[cc - j];
+                        const f32x2 w2 = a.win2[cc - j];
+                        h[j] = fma2(w2, v2, h[j]);
+                        hc[j] = fmaf(w, c, hc[j]);
+                    }
+            }
+#pragma unroll
+            for (int j = 0; j < kColsPer; ++j) {
+                float2 o;
+                unpack2(h[j], o.x, o.y);
+                s_hab[r * kRowStride + c0 + j] = o;
+                s_hc[r * kRowStride + c0 + j] = hc[j];
             }
         }
+        __syncthreads();
+        const int cc = tid % kTile, r0 = (tid / kTile) * kRowsPer;
+        const int px = bx + cc;
+        // the pixels of this thread, in flight during the vertical windows
+        float xv[kRowsPer], yv[kRowsPer];
 #pragma unroll
-        for (int mm = 0; mm < 3; ++mm)
+        for (int j = 0; j < kRowsPer; ++j) {
+            const bool in = px < a.W && by + r0 + j < a.H;
+            const size_t at = ch * P + (size_t)(by + r0 + j) * a.W + px;
+            xv[j] = in ? a.img[at] : 0.f;
+            yv[j] = in ? a.target[at] : 0.f;
+        }
+        f32x2 acc[kRowsPer];
+        float accc[kRowsPer];
 #pragma unroll
-            for (int j = 0; j < kColsPer; ++j) s_h[mm][r][c0 + j] = h[mm][j];
-    }
-    __syncthreads();
-        {
-            const int cc = tid % kTile, r0 = (tid / kTile) * kRowsPer;
-            float acc[3][kRowsPer];
+        for (int j = 0; j < kRowsPer; ++j) {
+            acc[j] = 0;
+            accc[j] = 0.f;
+        }
 #pragma unroll
-            for (int mm = 0; mm < 3; ++mm) {
+        for (int rr = 0; rr < kRowsPer + kWin - 1; ++rr) {
+            const float2 v = s_hab[(r0 + rr) * kRowStride + cc];
+            const float c = s_hc[(r0 + rr) * kRowStride + cc];
+            const f32x2 v2 = pack2(v.x, v.y);
 #pragma unroll
-                for (int j = 0; j < kRowsPer; ++j) acc[mm][j] = 0.f;
-#pragma unroll
-                for (int rr = 0; rr < kRowsPer + kWin - 1; ++rr) {
-                    const float v = s_h[mm][r0 + rr][cc];
-#pragma unroll
-                    for (int j = 0; j < kRowsPer; ++j)
-                        if (rr - j >= 0 && rr - j < kWin) acc[mm][j] += w[rr - j] * v;
+            for (int j = 0; j < kRowsPer; ++j)
+                if (rr - j >= 0 && rr - j < kWin) {
+                    const float w = a.win[rr - j];
+                    const f32x2 w2 = a.win2[rr - j];
+                    acc[j] = fma2(w2, v2, acc[j]);
+                    accc[j] = fmaf(w, c, accc[j]);
                 }
-            }
+        }
 #pragma unroll
-            for (int j = 0; j < kRowsPer; ++j) {
-                const int r = r0 + j;
-                const int px = bx + cc, py = by + r;
-                if (px >= a.W || py >= a.H) continue;
-                const size_t q = (size_t)py * a.W + px;
-                const float xv = a.img[ch * P + q], yv = a.target[ch * P + q];
-                const float d = xv - yv;
-                const float sgn = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
-                const float dssim = acc[0][j] + 2.f * xv * acc[1][j] + yv * acc[2][j];
-                a.dL_dimg[ch * P + q] = (1.f - a.lambda) * invN * sgn - a.lambda * invN * dssim;
-            }
+        for (int j = 0; j < kRowsPer; ++j) {
+            const int py = by + r0 + j;
+            if (px >= a.W || py >= a.H) continue;
+            const float d = xv[j] - yv[j];
+            const float sgn = d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f);
+            float wa, wb;
+            unpack2(acc[j], wa, wb);
+            const float dssim = wa + 2.f * xv[j] * wb + yv[j] * accc[j];
+            a.dL_dimg[ch * P + (size_t)py * a.W + px] = (1.f - a.lambda) * invN * sgn - a.lambda * invN * dssim;
         }
     }
 }
@@ -311,13 +378,21 @@ extern "C" gs_status gs_loss_l1_dssim(const float* img, const float* target, int
     a.H = height;
     a.lambda = lambda;
     a.done = reinterpret_cast<unsigned int*>(base);
-    a.coef = reinterpret_cast<float*>(base + 256);
+    a.coef_ab = reinterpret_cast<float2*>(base + 256);
+    a.coef_c = reinterpret_cast<float*>(base + 256) + 6 * P;
+    double win[kWin], sum = 0.0;
+    for (int k = 0; k < kWin; ++k) sum += win[k] = std::exp(-(double)((k - kHalf) * (k - kHalf)) / (2.0 * 1.5 * 1.5));
+    for (int k = 0; k < kWin; ++k) {
+        a.win[k] = (float)(win[k] / sum);
+        const float pair[2] = {a.win[k], a.win[k]};
+        std::memcpy(&a.win2[k], pair, sizeof(pair));
+    }
     a.partial = reinterpret_cast<double*>(base + 256 + ((9 * P * sizeof(float) + 255) / 256) * 256);
     a.out_loss = out_loss;
     a.dL_dimg = dL_dimg;
     if (cudaMemsetAsync(a.done, 0, sizeof(unsigned int), s) != cudaSuccess) return GS_ERR_CUDA;
     const dim3 grid((width + kTile - 1) / kTile, (height + kTile - 1) / kTile);
-    k_ssim_forward<<<grid, 256, 0, s>>>(a);
-    k_ssim_backward<<<grid, 256, 0, s>>>(a);
+    k_ssim_forward<<<grid, kLossThreads, 0, s>>>(a);
+    k_ssim_backward<<<grid, kLossThreads, 0, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }
