@@ -14,6 +14,8 @@
 //   -> dL/dM = (J W)^T dL/dV -> (s, R) -> q_hat -> q (normalisation Jacobian);
 //   dL/d(J W) -> dL/dJ -> dL/dt; dL/dmean2D -> dL/dt; dL/dt -> dL/dmu = W^T dL/dt;
 //   dL/drgb (clamp mask) -> dL/dSH = Y dL/drgb and -> dL/d dir -> dL/dmu.
+#include <algorithm>
+
 #include "gs_device.cuh"
 #include "gs_kernels.h"
 
@@ -354,6 +356,8 @@ __device__ __forceinline__ void bwd_view(const PreprocessBwdArgs& a, int i, cons
 // scene): the gradients of all the group's views are summed in registers and written once
 // (or added to the output when accumulating).  Group g owns blocks [block_base[g],
 // block_base[g+1]) and frames [frame_begin[g], frame_begin[g+1]).
+constexpr int kStageFloats = 48;   // longest row staged: 256 rows fill 48 KB
+
 template <int DEG, bool VEC, int MAXF, bool ISO>
 __global__ void __launch_bounds__(256) k_preprocess_backward_t(const __grid_constant__ BwdPlan<MAXF> m) {
     constexpr int D = (DEG + 1) * (DEG + 1);
@@ -369,10 +373,25 @@ __global__ void __launch_bounds__(256) k_preprocess_backward_t(const __grid_cons
         __syncthreads();
     }
     const PreprocessBwdArgs& a = MAXF == 1 ? m.a[0] : s_args[0];   // Gaussians and outputs shared by the group
-    const int i = (int)(blockIdx.x - m.block_base[g]) * blockDim.x + threadIdx.x;
-    if (i >= a.n) return;
-    float* gsh = a.g_sh + (size_t)i * a.sh_stride * 3;
+    const int first = (int)(blockIdx.x - m.block_base[g]) * blockDim.x;   // the block's first Gaussian
+    const int i = first + threadIdx.x;
     const int row = a.sh_stride * 3;   // floats per Gaussian in the SH buffers
+    // Rows that are not whole 16-byte vectors (degrees 0 and 2) go through shared memory: the block's
+    // rows are one contiguous run, moved with consecutive lanes on consecutive words, where a row
+    // per thread left every 32-byte sector to eight instructions (500k Gaussians of degree 2: 76 us).
+    extern __shared__ __align__(16) float s_rows[];
+    const bool staged = !VEC && row <= kStageFloats;
+    const int run = min((int)blockDim.x, a.n - first) * row;
+    if (staged) {
+        const float* src = a.sh + (size_t)first * row;
+        const int quads = (reinterpret_cast<uintptr_t>(src) & 15) == 0 ? run / 4 : 0;
+        for (int k = threadIdx.x; k < quads; k += blockDim.x)
+            reinterpret_cast<float4*>(s_rows)[k] = reinterpret_cast<const float4*>(src)[k];
+        for (int k = 4 * quads + threadIdx.x; k < run; k += blockDim.x) s_rows[k] = src[k];
+        __syncthreads();
+    }
+    if (i >= a.n && !staged) return;
+    float* gsh = a.g_sh + (size_t)i * row;
     BwdAcc<DEG> acc;
 #pragma unroll
     for (int k = 0; k < 3; ++k) acc.gm[k] = acc.gs[k] = 0.f;
@@ -387,7 +406,7 @@ __global__ void __launch_bounds__(256) k_preprocess_backward_t(const __grid_cons
     const int nv = MAXF == 1 ? 1 : f1 - f0;   // a single frame: straight-line code
     for (int k = 0; k < nv; ++k) {
         const PreprocessBwdArgs& av = MAXF == 1 ? m.a[0] : s_args[k];
-        if (av.radius[i] <= 0) continue;
+        if (i >= a.n || av.radius[i] <= 0) continue;
         if (!any) {
             any = true;
             mu[0] = a.means[3 * i]; mu[1] = a.means[3 * i + 1]; mu[2] = a.means[3 * i + 2];
@@ -398,12 +417,36 @@ __global__ void __launch_bounds__(256) k_preprocess_backward_t(const __grid_cons
                 s[0] = a.scales[3 * i]; s[1] = a.scales[3 * i + 1]; s[2] = a.scales[3 * i + 2];
                 q = reinterpret_cast<const float4*>(a.quats)[i];
             }
-            load_sh<D, VEC>(a.sh + (size_t)i * row, f);
+            load_sh<D, VEC>(staged ? s_rows + threadIdx.x * row : a.sh + (size_t)i * row, f);
         }
         bwd_view<DEG>(av, i, mu, s, q, f, acc);
     }
+    if (staged) {
+        float* mine = s_rows + threadIdx.x * row;   // each thread read its row before it writes it
+        if (i < a.n) {
+#pragma unroll
+            for (int k = 0; k < 3 * D; ++k) mine[k] = acc.gsh[k];
+            for (int k = 3 * D; k < row; ++k) mine[k] = 0.f;
+        }
+        __syncthreads();
+        float* dst = a.g_sh + (size_t)first * row;
+        const int quads = (reinterpret_cast<uintptr_t>(dst) & 15) == 0 ? run / 4 : 0;
+        for (int k = threadIdx.x; k < quads; k += blockDim.x) {
+            float4 v = reinterpret_cast<const float4*>(s_rows)[k];
+            float4* d = reinterpret_cast<float4*>(dst) + k;
+            if (a.accumulate) {
+                const float4 o = *d;
+                v = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
+            }
+            *d = v;
+        }
+        for (int k = 4 * quads + threadIdx.x; k < run; k += blockDim.x) dst[k] = a.accumulate ? dst[k] + s_rows[k] : s_rows[k];
+        if (i >= a.n) return;
+    }
     if (!any && a.accumulate) return;   // no view saw it: nothing to add
-    if (VEC && NF % 8 == 0 && row % 8 == 0 && (reinterpret_cast<uintptr_t>(gsh) & 31u) == 0) {
+    if (staged) {
+        // written above
+    } else if (VEC && NF % 8 == 0 && row % 8 == 0 && (reinterpret_cast<uintptr_t>(gsh) & 31u) == 0) {
 #pragma unroll
         for (int k = 0; k < NF / 8; ++k) {
             float v[8];
@@ -500,16 +543,32 @@ void preprocess_deg(const Multi<PreprocessArgs, MAXF>& m, bool vec, cudaStream_t
     }
 }
 
-template <int DEG, int MAXF>
-void preprocess_bwd_deg(const BwdPlan<MAXF>& m, bool vec, cudaStream_t s) {
-    const dim3 grid(m.block_base[m.groups]);
-    if (m.a[0].cfg.isotropic) {
-        if (vec) k_preprocess_backward_t<DEG, true, MAXF, true><<<grid, 256, 0, s>>>(m);
-        else k_preprocess_backward_t<DEG, false, MAXF, true><<<grid, 256, 0, s>>>(m);
-    } else {
-        if (vec) k_preprocess_backward_t<DEG, true, MAXF, false><<<grid, 256, 0, s>>>(m);
-        else k_preprocess_backward_t<DEG, false, MAXF, false><<<grid, 256, 0, s>>>(m);
+template <typename M>
+cudaError_t launch_rows(void (*kernel)(M), dim3 grid, size_t smem, const M& m, cudaStream_t s) {
+    if (smem > 32 * 1024) {   // with the static argument copy of a batch it may pass 48 KB
+        const cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
     }
+    kernel<<<grid, 256, smem, s>>>(m);
+    return cudaGetLastError();
+}
+
+template <int DEG, int MAXF>
+cudaError_t preprocess_bwd_deg(const BwdPlan<MAXF>& m, bool vec, cudaStream_t s) {
+    const dim3 grid(m.block_base[m.groups]);
+    // shared memory for the groups whose rows are staged (with a batch's arguments beside it)
+    size_t smem = 0;
+    if (!vec)
+        for (int g = 0; g < m.groups; ++g) {
+            const int row = 3 * m.a[m.frame_begin[g]].sh_stride;
+            if (row <= kStageFloats) smem = std::max(smem, (size_t)256 * row * sizeof(float));
+        }
+    if (m.a[0].cfg.isotropic) {
+        if (vec) return launch_rows(k_preprocess_backward_t<DEG, true, MAXF, true>, grid, smem, m, s);
+        return launch_rows(k_preprocess_backward_t<DEG, false, MAXF, true>, grid, smem, m, s);
+    }
+    if (vec) return launch_rows(k_preprocess_backward_t<DEG, true, MAXF, false>, grid, smem, m, s);
+    return launch_rows(k_preprocess_backward_t<DEG, false, MAXF, false>, grid, smem, m, s);
 }
 
 }  // namespace
@@ -540,12 +599,11 @@ cudaError_t launch_preprocess_backward(BwdPlan<MAXF>& m, cudaStream_t s) {
     const PreprocessBwdArgs& a = m.a[0];
     const bool vec = sh_vectorisable(a.sh, a.sh_stride, a.g_sh);
     switch (a.sh_degree) {
-        case 0: preprocess_bwd_deg<0>(m, vec, s); break;
-        case 1: preprocess_bwd_deg<1>(m, vec, s); break;
-        case 2: preprocess_bwd_deg<2>(m, vec, s); break;
-        default: preprocess_bwd_deg<3>(m, vec, s); break;
+        case 0: return preprocess_bwd_deg<0>(m, vec, s);
+        case 1: return preprocess_bwd_deg<1>(m, vec, s);
+        case 2: return preprocess_bwd_deg<2>(m, vec, s);
+        default: return preprocess_bwd_deg<3>(m, vec, s);
     }
-    return cudaGetLastError();
 }
 
 template cudaError_t launch_preprocess<1>(Multi<PreprocessArgs, 1>&, cudaStream_t);
