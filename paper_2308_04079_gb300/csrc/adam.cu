@@ -133,7 +133,7 @@ extern "C" gs_status gs_adam_step(const gs_adam_group* groups, int count, float 
     a.c2 = (float)(1.0 - std::pow((double)beta2, step));
     if (a.base[count] == 0) return GS_OK;
     const unsigned long long blocks = a.base[count];
-    const int cap = persistent_grid((const void*)k_adam, 256) * 8;
+    const int cap = persistent_blocks<k_adam>(256) * 8;
     k_adam<<<(int)(blocks < (unsigned long long)cap ? blocks : cap), 256, 0, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? GS_OK : GS_ERR_CUDA;
 }

@@ -1316,7 +1316,7 @@ __global__ void k_sort_prepare(const __grid_constant__ Multi<SortPrepareArgs, MA
 template <int MAXF>
 cudaError_t launch_depth_hist(Multi<DepthHistArgs, MAXF>& m, cudaStream_t s) {
     // blocks per frame: 8 keys per thread, at most a persistent grid each
-    const int cap = persistent_grid((const void*)k_depth_hist<MAXF>, 256);
+    const int cap = persistent_blocks<k_depth_hist<MAXF>>(256);
     m.base[0] = 0;
     for (int f = 0; f < m.frames; ++f) {
         const int b = std::min(std::max((m.a[f].n + 2047) / 2048, 1), cap);
@@ -1338,7 +1338,7 @@ cudaError_t launch_depth_small(const Multi<DepthSmallArgs, MAXF>& m, cudaStream_
 
 template <typename KeyT, int MAXF>
 cudaError_t launch_onesweep(const Multi<SortPassArgs<KeyT>, MAXF>& m, int max_chunks, cudaStream_t s) {
-    int grid = persistent_grid((const void*)k_onesweep<KeyT, MAXF>, kSortThreads);
+    int grid = persistent_blocks<k_onesweep<KeyT, MAXF>>(kSortThreads);
     if (max_chunks > 0 && grid > max_chunks) grid = max_chunks;
     k_onesweep<KeyT, MAXF><<<grid, kSortThreads, 0, s>>>(m);
     return cudaGetLastError();
@@ -1347,14 +1347,14 @@ cudaError_t launch_onesweep(const Multi<SortPassArgs<KeyT>, MAXF>& m, int max_ch
 template <int MAXF>
 cudaError_t launch_scan_tiles(const Multi<ScanArgs, MAXF>& m, bool key64, cudaStream_t s) {
     if (!key64) {   // the two-phase schedule: counting, scan and segment records in one pass
-        k_segments<MAXF><<<persistent_grid((const void*)k_segments<MAXF>, kDupThreads), kDupThreads, 0, s>>>(m);
+        k_segments<MAXF><<<persistent_blocks<k_segments<MAXF>>(kDupThreads), kDupThreads, 0, s>>>(m);
         return cudaGetLastError();
     }
     // KEY64: count, scan and write the segment records in three passes
-    k_count_tiles<true, MAXF><<<persistent_grid((const void*)k_count_tiles<true, MAXF>, kDupThreads), kDupThreads, 0,
+    k_count_tiles<true, MAXF><<<persistent_blocks<k_count_tiles<true, MAXF>>(kDupThreads), kDupThreads, 0,
                                 s>>>(m);
-    k_scan_pairs<MAXF><<<persistent_grid((const void*)k_scan_pairs<MAXF>, kDupThreads), kDupThreads, 0, s>>>(m);
-    k_write_segments<MAXF><<<persistent_grid((const void*)k_write_segments<MAXF>, kDupThreads), kDupThreads, 0, s>>>(
+    k_scan_pairs<MAXF><<<persistent_blocks<k_scan_pairs<MAXF>>(kDupThreads), kDupThreads, 0, s>>>(m);
+    k_write_segments<MAXF><<<persistent_blocks<k_write_segments<MAXF>>(kDupThreads), kDupThreads, 0, s>>>(
         m);
     return cudaGetLastError();
 }
@@ -1362,24 +1362,24 @@ cudaError_t launch_scan_tiles(const Multi<ScanArgs, MAXF>& m, bool key64, cudaSt
 template <int MAXF>
 cudaError_t launch_ranges(const Multi<RangesArgs, MAXF>& m, bool key64, cudaStream_t s) {
     if (key64)
-        k_ranges<true, MAXF><<<persistent_grid((const void*)k_ranges<true, MAXF>, 256), 256, 0, s>>>(m);
+        k_ranges<true, MAXF><<<persistent_blocks<k_ranges<true, MAXF>>(256), 256, 0, s>>>(m);
     else
-        k_ranges32<MAXF><<<persistent_grid((const void*)k_ranges32<MAXF>, 256), 256, 0, s>>>(m);
+        k_ranges32<MAXF><<<persistent_blocks<k_ranges32<MAXF>>(256), 256, 0, s>>>(m);
     return cudaGetLastError();
 }
 
 template <int MAXF>
 cudaError_t launch_emit(const Multi<EmitArgs, MAXF>& m, bool key64, cudaStream_t s) {
     if (key64)
-        k_emit<true, MAXF><<<persistent_grid((const void*)k_emit<true, MAXF>, kEmitThreads), kEmitThreads, 0, s>>>(m);
+        k_emit<true, MAXF><<<persistent_blocks<k_emit<true, MAXF>>(kEmitThreads), kEmitThreads, 0, s>>>(m);
     else
-        k_emit<false, MAXF><<<persistent_grid((const void*)k_emit<false, MAXF>, kEmitThreads), kEmitThreads, 0, s>>>(m);
+        k_emit<false, MAXF><<<persistent_blocks<k_emit<false, MAXF>>(kEmitThreads), kEmitThreads, 0, s>>>(m);
     return cudaGetLastError();
 }
 
 template <int MAXF>
 cudaError_t launch_sort_prepare(const Multi<SortPrepareArgs, MAXF>& m, cudaStream_t s) {
-    k_sort_prepare<MAXF><<<persistent_grid((const void*)k_sort_prepare<MAXF>, 256), 256, 0, s>>>(m);
+    k_sort_prepare<MAXF><<<persistent_blocks<k_sort_prepare<MAXF>>(256), 256, 0, s>>>(m);
     return cudaGetLastError();
 }
 
@@ -1409,7 +1409,7 @@ cudaError_t launch_clear(const Multi<ClearArgs, kMaxFrames>& m, cudaStream_t s) 
     for (int f = 0; f < m.frames; ++f)
         for (int r = 0; r < kClearRegions; ++r) words = std::max(words, m.a[f].ptr[r] ? m.a[f].words[r] : 0ull);
     const unsigned long long want = (words / 4 + 255) / 256;
-    const int grid = (int)std::max(1ull, std::min(want, (unsigned long long)persistent_grid((const void*)k_clear, 256)));
+    const int grid = (int)std::max(1ull, std::min(want, (unsigned long long)persistent_blocks<k_clear>(256)));
     k_clear<<<grid, 256, 0, s>>>(m);
     return cudaGetLastError();
 }

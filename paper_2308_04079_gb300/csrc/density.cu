@@ -509,7 +509,7 @@ extern "C" gs_status gs_densify(const gs_density_config* dc, int n, int sh_float
     p.result = result;
     if (cudaMemsetAsync(scratch, 0, zeroed, s) != cudaSuccess) return GS_ERR_CUDA;
     const int chunks = (n + kDensChunk - 1) / kDensChunk;
-    const int pcap = persistent_grid((const void*)k_densify_plan, kPlanThreads);
+    const int pcap = persistent_blocks<k_densify_plan>(kPlanThreads);
     k_densify_plan<<<chunks < pcap ? chunks : pcap, kPlanThreads, 0, s>>>(p);
     if (cudaGetLastError() != cudaSuccess) return GS_ERR_CUDA;
     if (out_capacity == 0) return GS_OK;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "gs.h"
 #include "gs_device.cuh"
 
@@ -336,8 +338,23 @@ struct TileOrderArgs {
 };
 
 // Host-side launchers (defined next to their kernels).  Each returns the launch status.
-// Persistent kernels size their grid as SM count x resident blocks per SM.
+// Persistent kernels size their grid as SM count x resident blocks per SM (asked of the runtime
+// once per kernel and device: the queries cost a launch-bound frame 10 of its 83 us of launches).
 int persistent_grid(const void* kernel, int threads);
+template <auto Kernel>
+int persistent_blocks(int threads) {
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= kDevices) return persistent_grid((const void*)Kernel, threads);
+    int blocks = known[dev].load(std::memory_order_relaxed);
+    if (blocks == 0) {
+        blocks = persistent_grid((const void*)Kernel, threads);
+        known[dev].store(blocks, std::memory_order_relaxed);
+    }
+    return blocks;
+}
 template <int MAXF> cudaError_t launch_preprocess(Multi<PreprocessArgs, MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_preprocess_backward(BwdPlan<MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_depth_small(const Multi<DepthSmallArgs, MAXF>& m, cudaStream_t s);

@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(kColThreads, 5) k_col_scatter(const __grid_con
 
 template <int MAXF>
 cudaError_t launch_col_count(const Multi<ColArgs, MAXF>& m, cudaStream_t s) {
-    k_col_count<MAXF><<<persistent_grid((const void*)k_col_count<MAXF>, kColThreads), kColThreads, 0, s>>>(m);
+    k_col_count<MAXF><<<persistent_blocks<k_col_count<MAXF>>(kColThreads), kColThreads, 0, s>>>(m);
     return cudaGetLastError();
 }
 
@@ -590,7 +590,7 @@ cudaError_t launch_tile_order(const Multi<TileOrderArgs, MAXF>& m, cudaStream_t 
 
 template <int MAXF>
 cudaError_t launch_col_scatter(const Multi<ColArgs, MAXF>& m, cudaStream_t s) {
-    k_col_scatter<MAXF><<<persistent_grid((const void*)k_col_scatter<MAXF>, kColThreads), kColThreads, 0, s>>>(m);
+    k_col_scatter<MAXF><<<persistent_blocks<k_col_scatter<MAXF>>(kColThreads), kColThreads, 0, s>>>(m);
     return cudaGetLastError();
 }
 
