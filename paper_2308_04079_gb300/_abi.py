@@ -243,6 +243,15 @@ def gs_read_status(frame: gs_frame, stream: int):
     return code, st
 
 
+def status_code(st: gs_device_status) -> int:
+    """The code gs_read_status returns for a status block (its device-side conditions)."""
+    for flag, code in ((FLAG_INTERNAL, GS_ERR_INTERNAL), (FLAG_TIMEOUT, GS_ERR_TIMEOUT),
+                       (FLAG_CAPACITY, GS_ERR_CAPACITY)):
+        if st.flags & flag:
+            return code
+    return GS_ERR_NUMERIC if st.num_nonfinite else GS_OK
+
+
 def gs_depth_order_static(n: int, depth: int, radius: int, order: int, status: int, stream: int) -> None:
     """Depth ordering with the library's static scratch (device pointers in, nothing
     allocated); see include/gs.h."""

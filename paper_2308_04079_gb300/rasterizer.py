@@ -46,12 +46,8 @@ def camera_struct(cam) -> abi.gs_camera:
     c = abi.gs_camera()
     c.width, c.height = int(cam.width), int(cam.height)
     c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
-    R = np.asarray(cam.R, dtype=np.float64).reshape(9)
-    t = np.asarray(cam.t, dtype=np.float64).reshape(3)
-    for k in range(9):
-        c.R[k] = float(R[k])
-    for k in range(3):
-        c.t[k] = float(t[k])
+    c.R[:] = np.asarray(cam.R, dtype=np.float64).reshape(9).tolist()
+    c.t[:] = np.asarray(cam.t, dtype=np.float64).reshape(3).tolist()
     c.near_z = float(getattr(cam, "near", 0.2))
     return c
 
@@ -67,7 +63,8 @@ def _stream() -> int:
 def _prep(t: torch.Tensor | None, align: int = 4) -> torch.Tensor | None:
     if t is None:
         return None
-    t = t.detach()
+    if t.requires_grad:
+        t = t.detach()
     if t.dtype != torch.float32:
         raise TypeError("rasterizer inputs must be float32")
     if not t.is_cuda:
@@ -121,6 +118,7 @@ class Frame:
         self.n = int(n)
         self.device = torch.device(device)
         self.cam = camera_struct(camera)
+        self._host_status = None    # pinned copy of the status block and the event of its read
         self._alloc(int(capacity) if capacity is not None else max(1 << 16, 4 * self.n))
 
     def _alloc(self, capacity: int):
@@ -135,7 +133,9 @@ class Frame:
 
     def set_camera(self, camera) -> None:
         """Another camera of the same image size (the workspace layout stays valid)."""
-        cam = camera_struct(camera)
+        self._set_camera(camera, camera_struct(camera))
+
+    def _set_camera(self, camera, cam: abi.gs_camera) -> None:
         if (cam.width, cam.height) != (self.cam.width, self.cam.height):
             raise ValueError("set_camera keeps the image size")
         self.camera, self.cam = camera, cam
@@ -211,17 +211,36 @@ class Frame:
 
     def ensure_binned(self, g: GaussianTensors) -> None:
         """preprocess + bin_sort; if the instance capacity was too small, grow it and redo."""
-        self.preprocess(g)
-        self.bin_sort()
-        code, st = self.status()
+        self._binned_then(g, None)
+
+    def _binned_then(self, g: GaussianTensors, then) -> None:
+        """ensure_binned with ``then()`` (launches that follow the binning on the stream) queued
+        before the host waits for the binning's status, so that the GPU has work while the host
+        reads it and prepares the next call.  After a capacity overflow the binning leaves every
+        tile empty: what ``then`` launched is harmless, and it is launched again after the redo."""
+        code, st = self._bin(g, then)
         if code == abi.GS_ERR_CAPACITY:
             self._alloc(int(st.num_instances * 1.25) + 1024)
-            self.preprocess(g)
-            self.bin_sort()
-            code, st = self.status()
+            code, st = self._bin(g, then)
         if code in (abi.GS_ERR_CAPACITY, abi.GS_ERR_TIMEOUT, abi.GS_ERR_INTERNAL):
             raise abi.GSError(code, "gs_bin_sort")
         self.last_status = st
+
+    def _bin(self, g: GaussianTensors, then):
+        self.preprocess(g)
+        self.bin_sort()
+        if then is None:
+            return self.status()
+        nbytes = ctypes.sizeof(abi.gs_device_status)
+        if self._host_status is None:
+            self._host_status = (torch.empty(nbytes, dtype=torch.uint8, pin_memory=True), torch.cuda.Event())
+        host, read = self._host_status
+        host.copy_(self.ws[self.layout.status:self.layout.status + nbytes], non_blocking=True)
+        read.record()
+        then()
+        read.synchronize()
+        st = abi.gs_device_status.from_buffer_copy(ctypes.string_at(host.data_ptr(), nbytes))
+        return abi.status_code(st), st
 
 
 def _gradients_struct(grads: dict) -> abi.gs_gradients:
@@ -305,7 +324,7 @@ def _frame_for(frame: Frame | None, n: int, camera, cfg, device) -> Frame:
     if (frame is None or frame.n != n or (frame.cam.width, frame.cam.height) != (cam.width, cam.height)
             or bytes(frame.cfg) != _cfg_bytes(cfg) or getattr(frame, "pending_backward", False)):
         return Frame(n, camera, cfg, device=device)
-    frame.set_camera(camera)
+    frame._set_camera(camera, cam)
     return frame
 
 
@@ -314,10 +333,9 @@ def render(g: GaussianTensors, camera, bg=(0.0, 0.0, 0.0), cfg=None, frame: Fram
     given ``frame`` is reused (with this camera) when its size and constants fit."""
     g = g.prepared()
     frame = _frame_for(frame, g.n, camera, cfg, g.means.device)
-    frame.ensure_binned(g)
-    img, T, last = frame.outputs()
-    frame.render_forward(bg, img, T, last)
-    return img, T, last, frame
+    outs = frame.outputs()
+    frame._binned_then(g, lambda: frame.render_forward(bg, *outs))
+    return (*outs, frame)
 
 
 class RasterizeFunction(torch.autograd.Function):
@@ -332,9 +350,8 @@ class RasterizeFunction(torch.autograd.Function):
         g = GaussianTensors(means, scales, quats, opacities, sh, settings["sh_degree"]).prepared()
         frame = _frame_for(settings.get("frame"), g.n, settings["camera"], settings.get("cfg"), g.means.device)
         settings["frame"] = frame
-        frame.ensure_binned(g)
         img, T, last = frame.outputs()
-        frame.render_forward(settings["bg"], img, T, last)
+        frame._binned_then(g, lambda: frame.render_forward(settings["bg"], img, T, last))
         frame.pending_backward = True
         ctx.frame = frame
         ctx.g = g
