@@ -238,6 +238,11 @@ bool sh_vec(const float* sh, int sh_stride, const float* gsh = nullptr) {
     return base && (3 * sh_stride) % 4 == 0;
 }
 
+bool same_gaussians(const gs_gaussians& a, const gs_gaussians& b) {
+    return a.means == b.means && a.scales == b.scales && a.quats == b.quats && a.opacities == b.opacities &&
+           a.sh == b.sh && a.n == b.n && a.sh_degree == b.sh_degree && a.sh_stride == b.sh_stride;
+}
+
 // Zeroes, per frame, the regions [ptr, ptr + words): cudaMemsetAsync for one frame, one kernel
 // for a batch.
 template <int MAXF>
@@ -271,34 +276,41 @@ gs_status preprocess_impl(const FrameSet<MAXF>& fs, const gs_gaussians* g, cudaS
     }
     gs_status st = clear_regions(fs, clr, s);
     if (st != GS_OK) return st;
-    // one launch per (SH degree, SH row alignment) class of frames
+    // one launch per (SH degree, SH row alignment) class of frames; frames that render the same
+    // Gaussians with the same kernel form a group
     bool done[MAXF] = {};
     for (int v0 = 0; v0 < fs.count; ++v0) {
         if (done[v0]) continue;
-        Multi<PreprocessArgs, MAXF> m;
-        m.frames = 0;
-        for (int v = v0; v < fs.count; ++v) {
-            if (done[v] || g[v].sh_degree != g[v0].sh_degree ||
-                sh_vec(g[v].sh, g[v].sh_stride) != sh_vec(g[v0].sh, g[v0].sh_stride))
+        PrePlan<MAXF> m;
+        m.groups = 0;
+        int nf = 0;
+        for (int u = v0; u < fs.count; ++u) {
+            if (done[u] || g[u].sh_degree != g[v0].sh_degree ||
+                sh_vec(g[u].sh, g[u].sh_stride) != sh_vec(g[v0].sh, g[v0].sh_stride))
                 continue;
-            done[v] = true;
-            const gs_frame* f = fs.f[v];
-            const Layout& L = fs.L[v];
-            void* ws = f->ws;
-            PreprocessArgs& a = m.a[m.frames++];
-            a.n = f->n;
-            a.means = g[v].means; a.scales = g[v].scales; a.quats = g[v].quats; a.opacities = g[v].opacities;
-            a.sh = g[v].sh;
-            a.sh_degree = g[v].sh_degree; a.sh_stride = g[v].sh_stride;
-            a.cam = cam_k(f, L);
-            a.cfg = cfg_k(f->cfg);
-            a.xy = at<float4>(ws, L.xy);
-            a.depth = at<float>(ws, L.depth);
-            a.conic_opacity = at<float4>(ws, L.conic);
-            a.rgb = at<float4>(ws, L.rgb);
-            a.radius = at<int>(ws, L.radius);
-            a.tau = at<float>(ws, L.tau);
-            a.status = &control_of(fs, v)->status;
+            m.frame_begin[m.groups++] = nf;
+            for (int v = u; v < fs.count; ++v) {
+                if (done[v] || !same_gaussians(g[u], g[v])) continue;
+                done[v] = true;
+                const gs_frame* f = fs.f[v];
+                const Layout& L = fs.L[v];
+                void* ws = f->ws;
+                PreprocessArgs& a = m.a[nf++];
+                a.n = f->n;
+                a.means = g[v].means; a.scales = g[v].scales; a.quats = g[v].quats; a.opacities = g[v].opacities;
+                a.sh = g[v].sh;
+                a.sh_degree = g[v].sh_degree; a.sh_stride = g[v].sh_stride;
+                a.cam = cam_k(f, L);
+                a.cfg = cfg_k(f->cfg);
+                a.xy = at<float4>(ws, L.xy);
+                a.depth = at<float>(ws, L.depth);
+                a.conic_opacity = at<float4>(ws, L.conic);
+                a.rgb = at<float4>(ws, L.rgb);
+                a.radius = at<int>(ws, L.radius);
+                a.tau = at<float>(ws, L.tau);
+                a.status = &control_of(fs, v)->status;
+            }
+            m.frame_begin[m.groups] = nf;
         }
         if (launch_preprocess(m, s) != cudaSuccess) return GS_ERR_CUDA;
     }
@@ -702,11 +714,6 @@ gs_status render_backward_tiles_impl(const FrameSet<MAXF>& fs, const float* bg, 
     gs_status st = clear_regions(fs, clr, s);
     if (st != GS_OK) return st;
     return ok(launch_render_backward(m, s));
-}
-
-bool same_gaussians(const gs_gaussians& a, const gs_gaussians& b) {
-    return a.means == b.means && a.scales == b.scales && a.quats == b.quats && a.opacities == b.opacities &&
-           a.sh == b.sh && a.n == b.n && a.sh_degree == b.sh_degree && a.sh_stride == b.sh_stride;
 }
 
 bool same_gradients(const gs_gradients& a, const gs_gradients& b) {

@@ -78,8 +78,6 @@ __device__ __forceinline__ float hw_rcp(float x) {
     return y;
 }
 
-__device__ __forceinline__ int floor_div(int a, int b) { return (a >= 0) ? a / b : -((-a + b - 1) / b); }
-
 __device__ __forceinline__ int clampi(int x, int lo, int hi) { return x < lo ? lo : (x > hi ? hi : x); }
 
 // Exponent of the 2D Gaussian at offset d = pixel centre - mean:
@@ -167,14 +165,16 @@ __device__ __forceinline__ int df_floor(float hi, float lo) {
 
 // Tile rectangle [x0, x1) x [y0, y1) of a splat with screen mean (u, v) and integer radius r:
 // x0 = floor((u - r) / tile_w), x1 = floor((u + r) / tile_w) + 1, clamped to the tile grid.
-// r is an integer, so floor((u -/+ r) / tile) = floor_div(floor(u) -/+ r, tile) exactly.
+// r is an integer, so floor((u -/+ r) / tile) = floor((floor(u) -/+ r) / tile) exactly, an arithmetic
+// shift.
 // The mean is the double-float m = (u_hi, v_hi, u_lo, v_lo).
 __device__ __forceinline__ bool tile_rect(float4 m, int r, const CamK& c, int& x0, int& x1, int& y0, int& y1) {
     const int fu = df_floor(m.x, m.z), fv = df_floor(m.y, m.w);
-    x0 = clampi(floor_div(fu - r, c.tile_w), 0, c.tiles_x);
-    x1 = clampi(floor_div(fu + r, c.tile_w) + 1, 0, c.tiles_x);
-    y0 = clampi(floor_div(fv - r, c.tile_h), 0, c.tiles_y);
-    y1 = clampi(floor_div(fv + r, c.tile_h) + 1, 0, c.tiles_y);
+    const int lw = c.tile_w == 16 ? 4 : 3, lh = c.tile_h == 16 ? 4 : 3;   // tile sides are 8 or 16
+    x0 = clampi((fu - r) >> lw, 0, c.tiles_x);
+    x1 = clampi(((fu + r) >> lw) + 1, 0, c.tiles_x);
+    y0 = clampi((fv - r) >> lh, 0, c.tiles_y);
+    y1 = clampi(((fv + r) >> lh) + 1, 0, c.tiles_y);
     return x0 < x1 && y0 < y1;
 }
 

@@ -124,16 +124,21 @@ struct PreprocessBwdArgs {
     int accumulate;
 };
 
-// Per-Gaussian backward of a batch: frames grouped by the Gaussians they render (group g =
-// frames [frame_begin[g], frame_begin[g + 1]), all with the same Gaussians, gradient outputs
-// and accumulate flag); group g owns blocks [block_base[g], block_base[g + 1]).
-template <int MAXF>
-struct BwdPlan {
+// Per-Gaussian kernels of a batch: frames grouped by the Gaussians they render (group g =
+// frames [frame_begin[g], frame_begin[g + 1]), all with the same Gaussians and, in the backward,
+// the same gradient outputs and accumulate flag); group g owns blocks [block_base[g],
+// block_base[g + 1]).
+template <typename A, int MAXF>
+struct GroupPlan {
     int groups;
     uint32_t block_base[MAXF + 1];
     int frame_begin[MAXF + 1];
-    PreprocessBwdArgs a[MAXF];
+    A a[MAXF];
 };
+template <int MAXF>
+using PrePlan = GroupPlan<PreprocessArgs, MAXF>;
+template <int MAXF>
+using BwdPlan = GroupPlan<PreprocessBwdArgs, MAXF>;
 
 // Zeroing of up to kClearRegions buffers per frame in one launch (batches).
 constexpr int kClearRegions = 4;
@@ -355,7 +360,7 @@ int persistent_blocks(int threads) {
     }
     return blocks;
 }
-template <int MAXF> cudaError_t launch_preprocess(Multi<PreprocessArgs, MAXF>& m, cudaStream_t s);
+template <int MAXF> cudaError_t launch_preprocess(PrePlan<MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_preprocess_backward(BwdPlan<MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_depth_small(const Multi<DepthSmallArgs, MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_depth_hist(Multi<DepthHistArgs, MAXF>& m, cudaStream_t s);

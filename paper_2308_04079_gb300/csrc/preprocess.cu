@@ -144,90 +144,100 @@ __device__ __forceinline__ void ld_v8(const float* p, float (&v)[8]) {
 // 6 blocks of 256 per SM (40 registers): config 3 (3M Gaussians) 0.157 -> 0.148 ms against the
 // 48-register build at 5 blocks; streaming or L2-only loads of the SH rows were slower (0.194,
 // 0.175 ms) and also slowed the backward, which re-reads the rows that stay in L2.
+// A batch's views of one scene go through one thread per Gaussian: its parameters and its SH row
+// come from L1 after the first view (as 16 sets of blocks, 16 views of 1M Gaussians read the 236 MB
+// of parameters 16 times: 796 -> 635 us; 4 scenes of 3 views 201 -> 176).  What bounds it then is
+// the instructions of the projection at half the warps (64 registers), not HBM.
 template <int DEG, bool VEC, int MAXF, bool ISO>
-__global__ void __launch_bounds__(256, 6) k_preprocess_t(const __grid_constant__ Multi<PreprocessArgs, MAXF> m) {
+__global__ void __launch_bounds__(256, MAXF == 1 ? 6 : 4) k_preprocess_t(const __grid_constant__ PrePlan<MAXF> m) {
     constexpr int D = (DEG + 1) * (DEG + 1);
-    const int f = find_frame<MAXF>(m.base, m.frames, blockIdx.x);   // frame f owns blocks [base[f], base[f+1])
-    // a batch reads its frame's arguments from a shared copy (generic loads otherwise)
-    __shared__ __align__(16) PreprocessArgs s_args;
+    const int g = find_frame<MAXF>(m.block_base, m.groups, blockIdx.x);
+    const int f0 = m.frame_begin[g], f1 = m.frame_begin[g + 1];
+    // a batch reads its group's arguments from a shared copy (generic loads otherwise)
+    __shared__ __align__(16) PreprocessArgs s_args[MAXF > 1 ? MAXF : 1];
     if (MAXF > 1) {
-        for (int k = threadIdx.x; k < (int)(sizeof(PreprocessArgs) / 4); k += blockDim.x)
-            reinterpret_cast<uint32_t*>(&s_args)[k] = reinterpret_cast<const uint32_t*>(&m.a[f])[k];
+        const int words = (int)(sizeof(PreprocessArgs) / 4) * (f1 - f0);
+        for (int k = threadIdx.x; k < words; k += blockDim.x)
+            reinterpret_cast<uint32_t*>(s_args)[k] = reinterpret_cast<const uint32_t*>(&m.a[f0])[k];
         __syncthreads();
     }
-    const PreprocessArgs& a = MAXF == 1 ? m.a[0] : s_args;
-    const int i = (int)(blockIdx.x - m.base[f]) * blockDim.x + threadIdx.x;
-    bool visible = false;
-    if (i < a.n) {
-        const CamK& c = a.cam;
-        const float mu[3] = {a.means[3 * i], a.means[3 * i + 1], a.means[3 * i + 2]};
-        // ISO (the isotropic ablation of Sec. 7.3): one scale for all axes and no rotation
-        const float s0 = ISO ? a.scales[i] : a.scales[3 * i];
-        const float s[3] = {s0, ISO ? s0 : a.scales[3 * i + 1], ISO ? s0 : a.scales[3 * i + 2]};
-        const float4 q = ISO ? make_float4(1.f, 0.f, 0.f, 0.f) : reinterpret_cast<const float4*>(a.quats)[i];
-        const float o = a.opacities[i];
-        const bool finite = finite3(mu) && finite3(s) && isfinite(q.x) && isfinite(q.y) && isfinite(q.z) &&
-                            isfinite(q.w) && isfinite(o);
-        int radius = 0;
-        float4 xy = make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 co = make_float4(0.f, 0.f, 0.f, 0.f);
-        float4 rgb = make_float4(0.f, 0.f, 0.f, 0.f);
-        float depth = 0.f;
-        Proj p;
-        if (!finite) {
-            atomicAdd(&a.status->num_nonfinite, 1u);
-        } else if (project_mean(mu, c, p) && (q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w) > 0.f) {
-            project_cov(s, q, c, a.cfg.dilation, p);
-            if (p.det > 0.f) {
-                // Cholesky factor of the conic (see splat_power).
-                co = make_float4(sqrtf(p.C / p.det), -p.B / sqrtf(p.C * p.det), 1.0f / sqrtf(p.C), o);
-                const float m = 0.5f * (p.A + p.C);
-                const float h = 0.5f * (p.A - p.C);
-                const float lam = m + sqrtf(h * h + p.B * p.B);
-                const float rr = a.cfg.extent * sqrtf(lam);
-                radius = rr >= (float)a.cfg.radius_max ? a.cfg.radius_max : (int)ceilf(rr);
-                xy = make_float4(p.u.hi, p.v.hi, p.u.lo, p.v.lo);
-                int x0, x1, y0, y1;
-                if (!tile_rect(xy, radius, c, x0, x1, y0, y1)) radius = 0;
-                depth = p.tz;
-            }
-        }
-        if (radius > 0) {
-            // View-dependent colour from the SH coefficients.
-            float dx = mu[0] - c.campos[0], dy = mu[1] - c.campos[1], dz = mu[2] - c.campos[2];
-            const float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
-            dx *= inv; dy *= inv; dz *= inv;
-            float Y[16];
-            sh_basis(DEG, dx, dy, dz, Y);
-            float f[4 * ((3 * D + 3) / 4)];
-            load_sh<D, VEC>(a.sh + (size_t)i * a.sh_stride * 3, f);
-            float r = 0.f, g = 0.f, b = 0.f;
-#pragma unroll
-            for (int k = 0; k < D; ++k) {
-                r += f[3 * k] * Y[k];
-                g += f[3 * k + 1] * Y[k];
-                b += f[3 * k + 2] * Y[k];
-            }
-            if (!(isfinite(r) && isfinite(g) && isfinite(b))) {
+    const PreprocessArgs& a0 = MAXF == 1 ? m.a[0] : s_args[0];   // Gaussians shared by the group
+    const int i = (int)(blockIdx.x - m.block_base[g]) * blockDim.x + threadIdx.x;
+    const int n = a0.n, nv = MAXF == 1 ? 1 : f1 - f0;   // a single frame: straight-line code
+    for (int v = 0; v < nv; ++v) {
+        const PreprocessArgs& a = MAXF == 1 ? m.a[0] : s_args[v];
+        bool visible = false;
+        if (i < n) {
+            const CamK& c = a.cam;
+            const float mu[3] = {a.means[3 * i], a.means[3 * i + 1], a.means[3 * i + 2]};
+            // ISO (the isotropic ablation of Sec. 7.3): one scale for all axes and no rotation
+            const float s0 = ISO ? a.scales[i] : a.scales[3 * i];
+            const float s[3] = {s0, ISO ? s0 : a.scales[3 * i + 1], ISO ? s0 : a.scales[3 * i + 2]};
+            const float4 q = ISO ? make_float4(1.f, 0.f, 0.f, 0.f) : reinterpret_cast<const float4*>(a.quats)[i];
+            const float o = a.opacities[i];
+            const bool finite = finite3(mu) && finite3(s) && isfinite(q.x) && isfinite(q.y) && isfinite(q.z) &&
+                                isfinite(q.w) && isfinite(o);
+            int radius = 0;
+            float4 xy = make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 co = make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 rgb = make_float4(0.f, 0.f, 0.f, 0.f);
+            float depth = 0.f;
+            Proj p;
+            if (!finite) {
                 atomicAdd(&a.status->num_nonfinite, 1u);
-                radius = 0;
-            } else {
-                const uint32_t mask = (r < 0.f ? 1u : 0u) | (g < 0.f ? 2u : 0u) | (b < 0.f ? 4u : 0u);
-                rgb = make_float4(fmaxf(r, 0.f), fmaxf(g, 0.f), fmaxf(b, 0.f), __uint_as_float(mask));
+            } else if (project_mean(mu, c, p) && (q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w) > 0.f) {
+                project_cov(s, q, c, a.cfg.dilation, p);
+                if (p.det > 0.f) {
+                    // Cholesky factor of the conic (see splat_power).
+                    co = make_float4(sqrtf(p.C / p.det), -p.B / sqrtf(p.C * p.det), 1.0f / sqrtf(p.C), o);
+                    const float m = 0.5f * (p.A + p.C);
+                    const float h = 0.5f * (p.A - p.C);
+                    const float lam = m + sqrtf(h * h + p.B * p.B);
+                    const float rr = a.cfg.extent * sqrtf(lam);
+                    radius = rr >= (float)a.cfg.radius_max ? a.cfg.radius_max : (int)ceilf(rr);
+                    xy = make_float4(p.u.hi, p.v.hi, p.u.lo, p.v.lo);
+                    int x0, x1, y0, y1;
+                    if (!tile_rect(xy, radius, c, x0, x1, y0, y1)) radius = 0;
+                    depth = p.tz;
+                }
             }
+            if (radius > 0) {
+                // View-dependent colour from the SH coefficients.
+                float dx = mu[0] - c.campos[0], dy = mu[1] - c.campos[1], dz = mu[2] - c.campos[2];
+                const float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
+                dx *= inv; dy *= inv; dz *= inv;
+                float Y[16];
+                sh_basis(DEG, dx, dy, dz, Y);
+                float f[4 * ((3 * D + 3) / 4)];
+                load_sh<D, VEC>(a.sh + (size_t)i * a.sh_stride * 3, f);
+                float r = 0.f, g = 0.f, b = 0.f;
+#pragma unroll
+                for (int k = 0; k < D; ++k) {
+                    r += f[3 * k] * Y[k];
+                    g += f[3 * k + 1] * Y[k];
+                    b += f[3 * k + 2] * Y[k];
+                }
+                if (!(isfinite(r) && isfinite(g) && isfinite(b))) {
+                    atomicAdd(&a.status->num_nonfinite, 1u);
+                    radius = 0;
+                } else {
+                    const uint32_t mask = (r < 0.f ? 1u : 0u) | (g < 0.f ? 2u : 0u) | (b < 0.f ? 4u : 0u);
+                    rgb = make_float4(fmaxf(r, 0.f), fmaxf(g, 0.f), fmaxf(b, 0.f), __uint_as_float(mask));
+                }
+            }
+            visible = radius > 0;
+            a.xy[i] = xy;
+            a.depth[i] = depth;
+            a.conic_opacity[i] = co;
+            a.rgb[i] = rgb;
+            a.radius[i] = radius;
+            // alpha >= alpha_min  <=>  d^T Q d <= 2 ln(o / alpha_min): the level the binning
+            // stage intersects with each tile row (reach_setup).
+            a.tau[i] = visible ? 2.0f * (logf(o) - logf(a.cfg.alpha_min)) : 0.0f;
         }
-        visible = radius > 0;
-        a.xy[i] = xy;
-        a.depth[i] = depth;
-        a.conic_opacity[i] = co;
-        a.rgb[i] = rgb;
-        a.radius[i] = radius;
-        // alpha >= alpha_min  <=>  d^T Q d <= 2 ln(o / alpha_min): the level the binning
-        // stage intersects with each tile row (reach_setup).
-        a.tau[i] = visible ? 2.0f * (logf(o) - logf(a.cfg.alpha_min)) : 0.0f;
+        const uint32_t vis = __ballot_sync(0xffffffffu, visible);
+        if ((threadIdx.x & 31) == 0 && vis) atomicAdd(&a.status->num_visible, (uint32_t)__popc(vis));
     }
-    const uint32_t vis = __ballot_sync(0xffffffffu, visible);
-    if ((threadIdx.x & 31) == 0 && vis) atomicAdd(&a.status->num_visible, (uint32_t)__popc(vis));
 }
 
 // Gradient of one Gaussian from one view, added into the accumulators (the Gaussian's
@@ -532,8 +542,8 @@ bool sh_vectorisable(const float* sh, int sh_stride, const float* gsh = nullptr)
 }
 
 template <int DEG, int MAXF>
-void preprocess_deg(const Multi<PreprocessArgs, MAXF>& m, bool vec, cudaStream_t s) {
-    const dim3 grid(m.base[m.frames]);
+void preprocess_deg(const PrePlan<MAXF>& m, bool vec, cudaStream_t s) {
+    const dim3 grid(m.block_base[m.groups]);
     if (m.a[0].cfg.isotropic) {
         if (vec) k_preprocess_t<DEG, true, MAXF, true><<<grid, 256, 0, s>>>(m);
         else k_preprocess_t<DEG, false, MAXF, true><<<grid, 256, 0, s>>>(m);
@@ -573,12 +583,13 @@ cudaError_t preprocess_bwd_deg(const BwdPlan<MAXF>& m, bool vec, cudaStream_t s)
 
 }  // namespace
 
-// Frames of one launch share the SH degree and the SH row alignment; the caller groups them.
+// Groups of one launch share the SH degree and the SH row alignment; the caller groups them.
 template <int MAXF>
-cudaError_t launch_preprocess(Multi<PreprocessArgs, MAXF>& m, cudaStream_t s) {
-    m.base[0] = 0;
-    for (int f = 0; f < m.frames; ++f) m.base[f + 1] = m.base[f] + (uint32_t)((m.a[f].n + 255) / 256);
-    if (m.base[m.frames] == 0) return cudaSuccess;
+cudaError_t launch_preprocess(PrePlan<MAXF>& m, cudaStream_t s) {
+    m.block_base[0] = 0;
+    for (int g = 0; g < m.groups; ++g)
+        m.block_base[g + 1] = m.block_base[g] + (uint32_t)((m.a[m.frame_begin[g]].n + 255) / 256);
+    if (m.block_base[m.groups] == 0) return cudaSuccess;
     const PreprocessArgs& a = m.a[0];
     const bool vec = sh_vectorisable(a.sh, a.sh_stride);
     switch (a.sh_degree) {
@@ -606,8 +617,8 @@ cudaError_t launch_preprocess_backward(BwdPlan<MAXF>& m, cudaStream_t s) {
     }
 }
 
-template cudaError_t launch_preprocess<1>(Multi<PreprocessArgs, 1>&, cudaStream_t);
-template cudaError_t launch_preprocess<kMaxFrames>(Multi<PreprocessArgs, kMaxFrames>&, cudaStream_t);
+template cudaError_t launch_preprocess<1>(PrePlan<1>&, cudaStream_t);
+template cudaError_t launch_preprocess<kMaxFrames>(PrePlan<kMaxFrames>&, cudaStream_t);
 template cudaError_t launch_preprocess_backward<1>(BwdPlan<1>&, cudaStream_t);
 template cudaError_t launch_preprocess_backward<kMaxFrames>(BwdPlan<kMaxFrames>&, cudaStream_t);
 
