@@ -247,12 +247,10 @@ __device__ __forceinline__ float low(f32x2 v) {
 
 // Sum over the lanes of a group of 9 values by a transposed reduce-scatter: each round halves the
 // values a lane keeps (it sends the half its partner keeps and adds the half it receives).  The
-// totals of slots [first, first + n) of reduce_slots are left in out[0..1].
-template <int GL>
-__device__ __forceinline__ void group_reduce9(const float (&v)[9], int lane, float (&out)[2]) {
-    float a[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) a[i] = v[i];
+// totals of slots [first, first + n) of reduce_slots are left in a[.][0..1].
+// U sets at once, so that their shuffles overlap.
+template <int GL, int U>
+__device__ __forceinline__ void group_reduce9(float (&a)[U][9], int lane) {
     int n = 9;
 #pragma unroll
     for (int m = GL / 2; m > 0; m >>= 1) {
@@ -261,17 +259,18 @@ __device__ __forceinline__ void group_reduce9(const float (&v)[9], int lane, flo
 #pragma unroll
         for (int i = 0; i < 5; ++i) {
             if (i >= half) continue;
-            if (half + i < n) {
-                const float keep = hi ? a[half + i] : a[i], send = hi ? a[i] : a[half + i];
-                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
-            } else {   // the odd value: both sides keep its sum
-                a[i] += __shfl_xor_sync(0xffffffffu, a[i], m);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (half + i < n) {
+                    const float keep = hi ? a[u][half + i] : a[u][i], send = hi ? a[u][i] : a[u][half + i];
+                    a[u][i] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+                } else {   // the odd value: both sides keep its sum
+                    a[u][i] += __shfl_xor_sync(0xffffffffu, a[u][i], m);
+                }
             }
         }
         n = half;
     }
-    out[0] = a[0];
-    out[1] = a[1];
 }
 
 // Slots [first, first + n) whose totals group_reduce9 leaves in this lane (n <= 2; a slot is
@@ -736,17 +735,21 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
             if (LN::ONE_PATH || (int)flags < 0) blend(std::true_type{});
             else blend(std::false_type{});
             if (LIMIT && !__any_sync(full, any_grad)) continue;
+            float v[U][9];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const float q = qs[u], t0 = sum2(sums[u][0]), t1 = sum2(sums[u][1]), qt0 = q * t0;
-                const float v[9] = {t1, qt0, sum2(sums[u][2]), q * t1, q * qt0, es[u].ko * t0, sum2(sums[u][3]),
-                                    sum2(sums[u][4]), sum2(sums[u][5])};
-                float tot[2];
-                group_reduce9<LN::GL>(v, ln.lane, tot);
+                v[u][0] = t1; v[u][1] = qt0; v[u][2] = sum2(sums[u][2]);
+                v[u][3] = q * t1; v[u][4] = q * qt0; v[u][5] = es[u].ko * t0;
+                v[u][6] = sum2(sums[u][3]); v[u][7] = sum2(sums[u][4]); v[u][8] = sum2(sums[u][5]);
+            }
+            group_reduce9<LN::GL, U>(v, ln.lane);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
                 if (at[u] != 0xffffffffu) {
                     float* dst = grad2d + 12 * (size_t)(es[u].id & 0x7fffffffu) + slot0;
-                    if (nslots > 0) atomicAdd(dst, f0 * tot[0]);
-                    if (nslots > 1) atomicAdd(dst + 1, f1 * tot[1]);
+                    if (nslots > 0) atomicAdd(dst, f0 * v[u][0]);
+                    if (nslots > 1) atomicAdd(dst + 1, f1 * v[u][1]);
                 }
             }
         }
