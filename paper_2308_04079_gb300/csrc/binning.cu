@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256) k_depth_hist(const __grid_constant__ Mult
         const uint32_t v = (&s_hist[0][0])[k];
         if (v) atomicAdd(&a.hist[k], v);
     }
-    const int rows = (a.n + kSortTile - 1) / kSortTile;
+    const int rows = (a.n + kSortThreads * a.items - 1) / (kSortThreads * a.items);
     for (long long k = (long long)lblock * blockDim.x + threadIdx.x; k < (long long)rows * 256; k += stride)
         a.lookback_first[k] = 0;
 }
@@ -216,9 +216,9 @@ __global__ void __launch_bounds__(kSmallThreads) k_depth_small(const __grid_cons
 // ---------------------------------------------------------------------------------------
 // One LSD digit pass (8 bits at `shift`), stable.
 // ---------------------------------------------------------------------------------------
-template <typename KeyT, int MAXF>
+// FEW: 4, 8 or 16 keys per thread, chosen by the arguments; else 16 (12 for 64-bit keys).
+template <typename KeyT, int MAXF, bool FEW>
 __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const __grid_constant__ Multi<SortPassArgs<KeyT>, MAXF> m) {
-    constexpr int ITEMS = SortTile<KeyT>::items;
     constexpr int TILE = SortTile<KeyT>::keys;
     constexpr int WARPS = kSortThreads / 32;
     __shared__ __align__(16) KeyT s_keys[TILE];
@@ -234,18 +234,29 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const __grid_const
     // A batch reads its frame's arguments from a shared copy: loads through a pointer into the
     // parameter array would be generic loads, repeated after every global store.
     __shared__ __align__(16) SortPassArgs<KeyT> s_args;
-    __shared__ int s_argf;
+    __shared__ int s_argf, s_items;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t lt = lanemask_lt();
     if (tid < 32) {
-        uint32_t c = 0;
+        uint32_t cnt = 0, all = 0;
         if (tid < m.frames) {
             const SortPassArgs<KeyT>& af = m.a[tid];
-            uint32_t cnt = af.count_host;
-            if (af.count_dev) cnt = min(cnt, *af.count_dev);
-            c = (cnt + TILE - 1) / TILE;
+            cnt = all = af.count_host;
+            if (af.count_dev) {
+                all = *af.count_dev;   // of every frame, sorted by this pass or not: all passes agree
+                cnt = min(cnt, all);
+            }
         }
+        int n_items = SortTile<KeyT>::items;
+        if (FEW) {
+            unsigned long long sum = all;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            n_items = m.a[0].items ? m.a[0].items : sort_items(sum);
+            if (tid == 0) s_items = n_items;
+        }
+        const uint32_t c = (cnt + kSortThreads * n_items - 1) / (kSortThreads * n_items);
         const uint32_t inc = warp_inclusive_scan<uint32_t>(c);
         if (tid < m.frames) s_base[tid + 1] = inc;
         if (tid == 0) {
@@ -256,6 +267,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const __grid_const
     }
     __syncthreads();
     const uint32_t total = s_base[m.frames];
+    const int items = FEW ? s_items : SortTile<KeyT>::items;   // keys per thread
     for (;;) {
         if (tid == 0) s_chunk = atomicAdd(m.a[0].chunk_counter, 1u);
         for (int k = tid; k < WARPS * 256; k += kSortThreads) (&s_hist[0][0])[k] = 0;
@@ -265,7 +277,10 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const __grid_const
         int f = 0;
         if (MAXF > 1)
             while (f + 1 < m.frames && s_base[f + 1] <= g) ++f;
-        auto body = [&](const SortPassArgs<KeyT>& a) {
+        // the number of keys per thread is a constant of the code: a loop with a run-time bound ranks
+        // and loads its keys one after another (3M keys: 40 -> 55 us a pass)
+        auto body = [&](const SortPassArgs<KeyT>& a, auto items_c) {
+        constexpr int ITEMS = decltype(items_c)::value;
         const uint32_t chunk = g - s_base[f];
         uint32_t count = a.count_host;
         if (a.count_dev) count = min(count, *a.count_dev);
@@ -275,7 +290,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const __grid_const
             if (tid == 0) s_frame = f;
         }
         if (a.lookback_next) a.lookback_next[(size_t)chunk * 256 + tid] = 0;
-        const uint32_t wbase = chunk * TILE + warp * 32 * ITEMS;
+        const uint32_t wbase = (chunk * kSortThreads + warp * 32) * ITEMS;
 
         KeyT key[ITEMS];
         uint32_t pos_local[ITEMS];
@@ -398,13 +413,22 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const __grid_const
             if (dest < count) {
                 a.keys_out[dest] = kk;
                 a.vals_out[dest] = s_vals[s];
-            } else if (GS_DEBUG && chunk * (uint32_t)TILE + s < count) {   // a real key: padding sorts last
+            } else if (GS_DEBUG && chunk * (uint32_t)(kSortThreads * ITEMS) + s < count) {   // a real key: padding sorts last
                 debug_fail(a.status);
             }
         }
         };
+        auto run = [&](const SortPassArgs<KeyT>& a) {
+            if constexpr (FEW) {
+                if (items == 16) body(a, std::integral_constant<int, 16>{});
+                else if (items == 8) body(a, std::integral_constant<int, 8>{});
+                else body(a, std::integral_constant<int, kSortMinItems>{});
+            } else {
+                body(a, std::integral_constant<int, SortTile<KeyT>::items>{});
+            }
+        };
         if constexpr (MAXF == 1) {
-            body(m.a[0]);
+            run(m.a[0]);
         } else {
             if (f != s_argf) {   // block-uniform
                 for (int k = tid; k < (int)(sizeof(SortPassArgs<KeyT>) / 4); k += kSortThreads)
@@ -412,7 +436,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const __grid_const
                 __syncthreads();
                 if (tid == 0) s_argf = f;
             }
-            body(s_args);
+            run(s_args);
         }
         __syncthreads();
     }
@@ -1019,7 +1043,10 @@ __global__ void __launch_bounds__(kDupThreads) k_segments(const __grid_constant_
             // the first record it covers (the number of records is known only at the end)
             if (a.row_passes) {
                 const unsigned long long end_s = min(base_s + blk_s, cap);
+                constexpr uint32_t least = kSortThreads * kSortMinItems;
                 for (unsigned long long r = (base_s + kSortTile - 1) / kSortTile; r * kSortTile < end_s; ++r)
+                    a.row_lb[r * 256 + tid] = 0u;
+                for (unsigned long long r = (base_s + least - 1) / least; r <= kSortFewChunks && r * least < end_s; ++r)
                     a.row_lb[r * 256 + tid] = 0u;
                 for (unsigned long long r = (base_s + kColChunk - 1) / kColChunk; r * kColChunk < end_s; ++r)
                     a.col_lb[r * 256 + tid] = 0u;
@@ -1315,11 +1342,13 @@ __global__ void k_sort_prepare(const __grid_constant__ Multi<SortPrepareArgs, MA
 
 template <int MAXF>
 cudaError_t launch_depth_hist(Multi<DepthHistArgs, MAXF>& m, cudaStream_t s) {
-    // blocks per frame: 8 keys per thread, at most a persistent grid each
+    // blocks per frame: 8 keys per thread (fewer with the passes' keys per thread, so that a frame of
+    // 60k Gaussians has 118 blocks instead of 30), at most a persistent grid each
     const int cap = persistent_blocks<k_depth_hist<MAXF>>(256);
     m.base[0] = 0;
     for (int f = 0; f < m.frames; ++f) {
-        const int b = std::min(std::max((m.a[f].n + 2047) / 2048, 1), cap);
+        const int per = m.a[f].items * kSortThreads / 2;
+        const int b = std::min(std::max((m.a[f].n + per - 1) / per, 1), cap);
         m.base[f + 1] = m.base[f] + (uint32_t)(m.a[f].n > 0 ? b : 0);
     }
     if (m.base[m.frames] == 0) return cudaSuccess;
@@ -1338,9 +1367,12 @@ cudaError_t launch_depth_small(const Multi<DepthSmallArgs, MAXF>& m, cudaStream_
 
 template <typename KeyT, int MAXF>
 cudaError_t launch_onesweep(const Multi<SortPassArgs<KeyT>, MAXF>& m, int max_chunks, cudaStream_t s) {
-    int grid = persistent_blocks<k_onesweep<KeyT, MAXF>>(kSortThreads);
+    const bool few = sizeof(KeyT) == 4 && m.a[0].items != SortTile<KeyT>::items;
+    int grid = few ? persistent_blocks<k_onesweep<KeyT, MAXF, sizeof(KeyT) == 4>>(kSortThreads)
+                   : persistent_blocks<k_onesweep<KeyT, MAXF, false>>(kSortThreads);
     if (max_chunks > 0 && grid > max_chunks) grid = max_chunks;
-    k_onesweep<KeyT, MAXF><<<grid, kSortThreads, 0, s>>>(m);
+    if (few) k_onesweep<KeyT, MAXF, sizeof(KeyT) == 4><<<grid, kSortThreads, 0, s>>>(m);
+    else k_onesweep<KeyT, MAXF, false><<<grid, kSortThreads, 0, s>>>(m);
     return cudaGetLastError();
 }
 

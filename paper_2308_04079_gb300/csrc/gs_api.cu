@@ -97,7 +97,10 @@ bool make_layout(int n, int W, int H, uint64_t cap, const gs_raster_config* cfg,
     L->scan_lb_rows = (nn + kDupThreads - 1) / kDupThreads;
     L->scan_lb = take(L->scan_lb_rows * sizeof(unsigned long long));
     const size_t rows_n = (nn + kSortTile - 1) / kSortTile, rows_c = (cc + kSortTileMin - 1) / kSortTileMin;
-    L->sort_lb_rows = rows_n > rows_c ? rows_n : rows_c;
+    // (sorts of few keys take smaller chunks, at most kSortFewChunks of them)
+    const size_t least = (size_t)kSortThreads * kSortMinItems;
+    const size_t rows_few = std::min((std::max(nn, cc) + least - 1) / least, (size_t)kSortFewChunks + 1);
+    L->sort_lb_rows = std::max(std::max(rows_n, rows_c), rows_few);
     for (int k = 0; k < 2; ++k) L->sort_lb[k] = take(L->sort_lb_rows * 256 * sizeof(uint32_t));
     // ikey[1] / ival[1] also hold the segment records between the scan and the emit kernel:
     // first tiles and offsets (capacity + 1 entries) in ikey[1], Gaussian ids in ival[1].
@@ -360,6 +363,7 @@ gs_status key_sort(const FrameSet<MAXF>& fs, cudaStream_t s) {
             a.chunk_counter = &ctl0->counters[8 + p];
             a.status = &ctl->status;
             a.spin_limit = fs.f[v]->cfg.spin_limit;
+            a.items = SortTile<KeyT>::items;
         }
         if (launch_onesweep(m, 0, s) != cudaSuccess) return GS_ERR_CUDA;
         phase("instance radix pass", s);
@@ -415,7 +419,11 @@ gs_status tiles_by_radix(const FrameSet<MAXF>& fs, bool key64, cudaStream_t s) {
 template <int MAXF>
 gs_status tiles_by_rows(const FrameSet<MAXF>& fs, cudaStream_t s) {
     int max_passes = 0;
-    for (int v = 0; v < fs.count; ++v) max_passes = std::max(max_passes, fs.L[v].row_passes);
+    unsigned long long capacity = 0;
+    for (int v = 0; v < fs.count; ++v) {
+        max_passes = std::max(max_passes, fs.L[v].row_passes);
+        capacity += fs.f[v]->capacity;
+    }
     Control* ctl0 = control_of(fs, 0);
     for (int p = 0; p < max_passes; ++p) {
         Multi<SortPassArgs<uint32_t>, MAXF> m;
@@ -443,6 +451,7 @@ gs_status tiles_by_rows(const FrameSet<MAXF>& fs, cudaStream_t s) {
             a.chunk_counter = &ctl0->counters[8 + p];
             a.status = &ctl->status;
             a.spin_limit = fs.f[v]->cfg.spin_limit;
+            a.items = capacity > kSortFewCapacity ? SortTile<uint32_t>::items : 0;
         }
         if (launch_onesweep(m, 0, s) != cudaSuccess) return GS_ERR_CUDA;
         phase("row radix pass", s);
@@ -534,13 +543,16 @@ gs_status bin_sort_impl(const FrameSet<MAXF>& fs, cudaStream_t s) {
         Multi<DepthHistArgs, MAXF> h;
         h.frames = fs.count;
         int chunks = 0;
+        unsigned long long keys = 0;
+        for (int v = 0; v < fs.count; ++v) keys += (unsigned long long)fs.f[v]->n;
+        const int items = sort_items(keys), tile = kSortThreads * items;
         for (int v = 0; v < fs.count; ++v) {
             const Layout& L = fs.L[v];
             void* ws = fs.f[v]->ws;
             Control* ctl = control_of(fs, v);
             h.a[v] = DepthHistArgs{fs.f[v]->n, at<float>(ws, L.depth), at<int>(ws, L.radius), &ctl->hist_depth[0][0],
-                                   at<uint32_t>(ws, L.sort_lb[0]), &ctl->counters[31]};
-            chunks += (fs.f[v]->n + kSortTile - 1) / kSortTile;
+                                   at<uint32_t>(ws, L.sort_lb[0]), &ctl->counters[31], items};
+            chunks += (fs.f[v]->n + tile - 1) / tile;
         }
         if (launch_depth_hist(h, s) != cudaSuccess) return GS_ERR_CUDA;
         phase("depth histogram", s);
@@ -569,6 +581,7 @@ gs_status bin_sort_impl(const FrameSet<MAXF>& fs, cudaStream_t s) {
                 a.chunk_counter = &ctl0->counters[1 + p];
                 a.status = &ctl->status;
                 a.spin_limit = fs.f[v]->cfg.spin_limit;
+                a.items = items;
             }
             if (chunks > 0 && launch_onesweep(m, chunks, s) != cudaSuccess) return GS_ERR_CUDA;
             phase("depth radix pass", s);

@@ -35,6 +35,20 @@ struct SortTile {
 };
 constexpr int kSortTile = SortTile<uint32_t>::keys;            // 4096
 constexpr int kSortTileMin = SortTile<unsigned long long>::keys; // 3072
+// 32-bit keys per thread of a launch that sorts `keys` of them: 16, or fewer while that leaves no
+// more than kSortFewChunks chunks: a chunk's keys are ranked in series, so a pass over few chunks
+// takes the time of one.  Histogram + four depth passes, 16 keys per thread -> this rule, us: 60k
+// Gaussians 70 -> 47, 200k 75 -> 60, 500k 81 -> 79 (4 keys there: 85); the row pass over 131k records
+// 17 -> 14, over 651k 21 -> 19 (16 keys in the kernel that chooses: 25).
+constexpr uint32_t kSortFewChunks = 512;
+constexpr int kSortMinItems = 4;
+__host__ __device__ constexpr int sort_items(unsigned long long keys) {
+    return keys <= (1u << 18) ? kSortMinItems : keys <= (1u << 20) ? 8 : SortTile<uint32_t>::items;
+}
+static_assert((1u << 18) / (256 * kSortMinItems) <= kSortFewChunks && (1u << 20) / (256 * 8) <= kSortFewChunks, "look-back rows");
+// A row pass (its keys counted on the device) may choose at run time only where the capacities of
+// the launch allow few records; that kernel holds every variant and is 4-8 % slower at 16.
+constexpr unsigned long long kSortFewCapacity = 6000000;
 constexpr int kMaxKeyPasses = 8;
 constexpr int kMaxTilePasses = 3;   // tile ids below 2^24
 constexpr int kDepthPasses = 4;
@@ -154,6 +168,7 @@ struct DepthHistArgs {
     uint32_t* hist;            // [4][256]
     uint32_t* lookback_first;  // rows for the first depth pass
     uint32_t* num_visible;     // count of radius > 0 (zeroed)
+    int items;                 // keys per thread of the depth passes (SortPassArgs)
 };
 
 template <typename KeyT>
@@ -176,6 +191,8 @@ struct SortPassArgs {
     uint32_t* chunk_counter;   // zeroed
     gs_device_status* status;
     uint32_t spin_limit;       // look-back polls before giving up (kFlagTimeout)
+    int items;                 // 32-bit keys per thread, the same for all frames (launch_onesweep);
+                               // 0: sort_items of the launch's device-side counts
 };
 
 struct ScanArgs {

@@ -84,7 +84,8 @@ extern "C" gs_status gs_depth_order_static(int n, const float* depth, const int*
 
     Multi<DepthHistArgs, 1> h;
     h.frames = 1;
-    h.a[0] = DepthHistArgs{n, depth, radius, &sc->hist[0][0], sc->lookback[0], &status->num_visible};
+    h.a[0] = DepthHistArgs{n, depth, radius, &sc->hist[0][0], sc->lookback[0], &status->num_visible,
+                             SortTile<uint32_t>::items};
     if (launch_depth_hist(h, s) != cudaSuccess) return GS_ERR_CUDA;
     const int chunks = (n + kSortTile - 1) / kSortTile;
     for (int p = 0; p < kDepthPasses; ++p) {
@@ -109,6 +110,7 @@ extern "C" gs_status gs_depth_order_static(int n, const float* depth, const int*
         a.chunk_counter = &sc->counters[p];
         a.status = status;
         a.spin_limit = kSpinLimit;
+        a.items = SortTile<uint32_t>::items;
         if (launch_onesweep(m, chunks, s) != cudaSuccess) return GS_ERR_CUDA;
     }
     return GS_OK;

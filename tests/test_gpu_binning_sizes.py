@@ -1,6 +1,6 @@
 """The two-phase schedule changes its layout with the frame's size: a frame of at most 8,192
-Gaussians is depth-sorted by one block, and the column passes take 256 to 2,048 records per chunk
-by the number of records of the launch.  At the edges of these ranges the result is that of the
+Gaussians is depth-sorted by one block, the radix passes take 4, 8 or 16 keys per thread by the number
+of keys, and the column passes 256 to 2,048 records per chunk by the number of records of the launch.  At the edges of these ranges the result is that of the
 KEY64 schedule, which shares none of it, bit for bit."""
 import numpy as np
 import pytest
@@ -52,3 +52,22 @@ def test_column_chunk_sizes(n, W, H, rmax):
     for x, y in zip(a[2:], b[2:]):
         assert np.array_equal(x, y)
     print(f"n {n}: {a[1]} records, {a[0]} instances")
+
+
+@pytest.mark.parametrize("n", [1 << 18, (1 << 18) + 1, (1 << 20) - 3, (1 << 20) + 1])
+def test_depth_passes_where_the_keys_per_thread_change(n):
+    sp = _screen(160, n, 640, 480, 4, culled=0.3, ties=0.3)
+    a, b = (_binned(sp, 640, 480, mode, 6_000_000) for mode in ("two_phase", "key64"))
+    assert a[0] == b[0] and a[1] == b[1]
+    for x, y in zip(a[2:], b[2:]):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("capacity", [6_000_000, 6_000_001])
+def test_two_row_passes_in_either_kernel(capacity):
+    # over 256 tile rows: two row passes, with the keys per thread chosen on the device or fixed
+    sp = _screen(161, 60_000, 300, 4400, 60)
+    a, b = (_binned(sp, 300, 4400, mode, capacity) for mode in ("two_phase", "key64"))
+    assert a[0] == b[0] and a[1] == b[1]
+    for x, y in zip(a[2:], b[2:]):
+        assert np.array_equal(x, y)
