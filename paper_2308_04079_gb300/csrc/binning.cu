@@ -17,8 +17,8 @@
 // Radix sort: one kernel per digit pass in the onesweep style (Merrill & Grimshaw's radix
 // sorting, single-pass with decoupled look-back): every block claims a 4096-key chunk from an
 // atomic counter (chunks are claimed in order, so a block only ever waits on chunks already
-// held by running blocks), ranks its keys with warp-private shared-memory digit counters and
-// __match_any_sync, publishes per-digit counts, resolves its global digit offsets by looking
+// held by running blocks), ranks its keys with warp-private shared-memory digit counters,
+// publishes per-digit counts, resolves its global digit offsets by looking
 // back over predecessor chunks (bounded spin), stages the keys in shared memory in local sorted
 // order and writes them out coalesced.  Digit histograms of every pass are computed up front
 // (fused into the kernel that produces the keys).
@@ -59,26 +59,31 @@ __global__ void __launch_bounds__(256) k_depth_hist(const __grid_constant__ Mult
     __shared__ uint32_t s_vis;
     if (threadIdx.x == 0) s_vis = 0;
     const int lane = threadIdx.x & 31;
-    const uint32_t lt = lanemask_lt();
     const int stride = nblocks * blockDim.x;
     uint32_t vis_count = 0;   // per warp (lane 0); one global atomic per block at the end
-    for (int base = lblock * blockDim.x; base < a.n; base += stride) {
-        const int i = base + threadIdx.x;
-        const bool valid = i < a.n;
-        uint32_t key = 0xFFFFFFFFu;
-        if (valid && a.radius[i] > 0) key = __float_as_uint(a.depth[i]);
-        // the two low bytes of the depth bits are spread (plain shared atomics rarely collide);
-        // the two high bytes repeat across a warp (one atomic per distinct digit)
+    // Bound by the loads' latency and the shared atomics.  One plain atomic per key and byte, also
+    // for the high bytes that repeat across a warp: finding the distinct digits first with
+    // __match_any_sync cost more than the collisions it saved (3M keys: 33 -> 26 us), and four
+    // keys' loads in flight per thread give the rest (26 -> 21 us; eight: 20, the stage unchanged).
+    constexpr int kLoads = 4;
+    for (long long base = (long long)lblock * blockDim.x + threadIdx.x; base - lane < a.n; base += (long long)kLoads * stride) {
+        int radius[kLoads];
+        float depth[kLoads];
 #pragma unroll
-        for (int p = 0; p < 2; ++p)
-            if (valid) atomicAdd(&s_hist[p][(key >> (8 * p)) & 0xFFu], 1u);
-#pragma unroll
-        for (int p = 2; p < 4; ++p) {
-            const uint32_t d = valid ? (key >> (8 * p)) & 0xFFu : 0x100u;
-            const uint32_t peers = __match_any_sync(0xffffffffu, d);
-            if (valid && (peers & lt) == 0) atomicAdd(&s_hist[p][d], (uint32_t)__popc(peers));
+        for (int u = 0; u < kLoads; ++u) {
+            const long long i = base + (long long)u * stride;
+            radius[u] = i < a.n ? a.radius[i] : 0;
+            depth[u] = i < a.n ? a.depth[i] : 0.f;
         }
-        vis_count += (uint32_t)__popc(__ballot_sync(0xffffffffu, valid && key != 0xFFFFFFFFu));
+#pragma unroll
+        for (int u = 0; u < kLoads; ++u) {
+            const uint32_t key = radius[u] > 0 ? __float_as_uint(depth[u]) : 0xFFFFFFFFu;
+            if (base + (long long)u * stride < a.n) {
+#pragma unroll
+                for (int p = 0; p < 4; ++p) atomicAdd(&s_hist[p][(key >> (8 * p)) & 0xFFu], 1u);
+            }
+            vis_count += (uint32_t)__popc(__ballot_sync(0xffffffffu, key != 0xFFFFFFFFu));
+        }
     }
     __syncthreads();
     if (lane == 0 && vis_count) atomicAdd(&s_vis, vis_count);
@@ -309,32 +314,43 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_onesweep(const __grid_const
         }
         // Warp-level stable ranking: lanes with equal digits are ordered by lane, items by i.
         uint32_t* wh = s_hist[warp];
+        // Lanes holding the same digit (`peers`), by one of two ways.  Spread digits: every lane sets
+        // its bit in the warp's word of its digit and reads the word back, at a cost that grows with
+        // the lanes per digit; __match_any_sync's grows with the distinct digits, and eight ballots
+        // cost as much as it does.  3M depth keys, us a pass: 47/41/39 with match_any, 38/30/29 with
+        // the words, but the top byte, of few values, 25 against 35: the host names such passes.
+        // Row bytes of 9M records: 90 -> 65.  A warp of one digit (culled keys) needs no words.
+        auto ranked = [&](auto peers_of, uint32_t* words) {
 #pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const uint32_t d = digit_of(key[i], a.shift, a.mask);
-            // lanes holding the same digit: __match_any_sync costs more the more distinct
-            // digits a warp holds, one ballot per digit bit costs the same for any keys; the
-            // host asks for ballots (as many as the pass's digits have bits) on passes whose
-            // digits are spread (the first tile pass)
-            uint32_t peers;
-            if (a.ballot_rank) {
-                peers = 0xffffffffu;
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    if (b < a.ballot_rank) {
-                        const uint32_t bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-                        peers &= ((d >> b) & 1u) ? bal : ~bal;
-                    }
+            for (int i = 0; i < ITEMS; ++i) {
+                const uint32_t d = digit_of(key[i], a.shift, a.mask);
+                const uint32_t peers = peers_of(d);
+                const uint32_t below = peers & lt;
+                const uint32_t prev = wh[d];
+                __syncwarp();
+                if (below == 0) {
+                    wh[d] = prev + (uint32_t)__popc(peers);
+                    if (words) words[d] = 0;
                 }
-            } else {
-                peers = __match_any_sync(0xffffffffu, d);
+                __syncwarp();
+                pos_local[i] = prev + (uint32_t)__popc(below);
             }
-            const uint32_t below = peers & lt;
-            const uint32_t prev = wh[d];
+        };
+        if (a.repeated) {
+            ranked([&](uint32_t d) { return __match_any_sync(0xffffffffu, d); }, nullptr);
+        } else {
+            // the words lie in s_keys, which the staging fills after the block's next barrier
+            static_assert(sizeof(s_keys) >= WARPS * 256 * sizeof(uint32_t), "words of the warps' digits");
+            uint32_t* const words = reinterpret_cast<uint32_t*>(s_keys) + warp * 256;
+#pragma unroll
+            for (int k = 0; k < 256; k += 32) words[k + lane] = 0;
             __syncwarp();
-            if (below == 0) wh[d] = prev + (uint32_t)__popc(peers);
-            __syncwarp();
-            pos_local[i] = prev + (uint32_t)__popc(below);
+            ranked([&](uint32_t d) {
+                if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) return 0xffffffffu;
+                atomicOr(&words[d], 1u << lane);
+                __syncwarp();
+                return words[d];
+            }, words);
         }
         __syncthreads();
         // Per digit (thread = digit): warp offsets, block count, block-local start.

@@ -183,8 +183,8 @@ struct SortPassArgs {
     uint32_t count_host;       // element count bound (capacity)
     int shift;                 // digit = (key >> shift) & mask
     uint32_t mask;
-    int ballot_rank;           // > 0: rank digits with that many ballots (every digit below
-                               // 2^ballot_rank; spread digits), 0: with match_any
+    int repeated;              // the digits repeat across a warp (few values): how lanes of one
+                               // digit find each other
     const uint32_t* hist;      // [256] digit counts of this pass
     uint32_t* lookback;        // [chunks][256], zeroed
     uint32_t* lookback_next;   // rows to zero for the next pass, or null
