@@ -14,7 +14,7 @@
 //   3. k_tile_scan: exclusive scan of the tile counts = the [start, end) range of every tile, and
 //      the render order of the tiles;
 //   4. k_col_scatter, per chunk: the records' instances, expanded in rounds of kRound, ranked
-//      stably by column (one ballot per digit bit, per-warp counters), staged in shared
+//      stably by column (lanes of one column meet in a word of shared memory, per-warp counters), staged in shared
 //      memory in column order and written to start(tile) + (the row's instances of that column
 //      in earlier chunks and rounds) + rank: every instance goes straight to its final slot.
 // Within a tile, instances keep the record order, which is the depth order: the result is
@@ -375,8 +375,11 @@ __global__ void __launch_bounds__(kColThreads, 5) k_col_scatter(const __grid_con
     __shared__ uint32_t s_offx[kColChunk + 1];        // first instance of the record in the chunk << 8 | column
     __shared__ uint16_t s_row[kColChunk];
     __shared__ uint32_t s_item[kRound + kRound / 32];  // column | record << 8 (padded), then staged Gaussians
-    __shared__ uint8_t s_col[kRound];                  // column of each staged instance
-    __shared__ uint32_t s_hist[kColWarps][256];
+    // counts of a round fit 16 bits (kRound), which leaves the shared memory of five blocks per SM
+    __shared__ __align__(4) uint16_t s_hist[kColWarps][256];
+    __shared__ uint32_t s_words[kColWarps][256];       // while ranking: the lanes of each column
+    uint8_t* const s_col = reinterpret_cast<uint8_t*>(s_words);   // then: column of each staged instance
+    static_assert(sizeof(s_words) >= kRound && kRound <= 65535, "staged columns, 16-bit counts");
     __shared__ uint32_t s_bstart[256], s_gbase[256], s_dst[256];
     __shared__ uint32_t s_scan[33];
     __shared__ uint32_t s_chunk;
@@ -462,7 +465,8 @@ __global__ void __launch_bounds__(kColThreads, 5) k_col_scatter(const __grid_con
                     // short rounds are spread over all threads and warps
                     const uint32_t tshare = (n + kColThreads - 1) / kColThreads;
                     const uint32_t wshare = tshare * 32u;
-                    for (int k = tid; k < kColWarps * 256; k += kColThreads) (&s_hist[0][0])[k] = 0;
+                    for (int k = tid; k < kColWarps * 128; k += kColThreads) reinterpret_cast<uint32_t*>(s_hist)[k] = 0;
+                    for (int k = tid; k < kColWarps * 256; k += kColThreads) (&s_words[0][0])[k] = 0;
                     // thread t expands instances [tshare t, tshare t + tshare) of the round: record
                     // by a search for the first, then a walk
                     {
@@ -495,7 +499,8 @@ __global__ void __launch_bounds__(kColThreads, 5) k_col_scatter(const __grid_con
                     __syncthreads();
                     // rank by column: warps in order, then items, then lanes (= instance order)
                     uint32_t it[kRoundPer], pos[kRoundPer];
-                    uint32_t* wh = s_hist[warp];
+                    uint16_t* wh = s_hist[warp];
+                    uint32_t* words = s_words[warp];
                     const uint32_t wbase = (uint32_t)warp * wshare;
 #pragma unroll
                     for (int i = 0; i < kRoundPer; ++i) {
@@ -505,16 +510,19 @@ __global__ void __launch_bounds__(kColThreads, 5) k_col_scatter(const __grid_con
                         const uint32_t qq = wbase + (uint32_t)i * 32 + (uint32_t)lane;
                         if (qq < n) it[i] = s_item[pad32(qq)];
                         const uint32_t d = it[i] & 0xFFu;
-                        uint32_t peers = 0xffffffffu;
-#pragma unroll
-                        for (int b = 0; b < 8; ++b) {   // all 8 bits: no branch per bit
-                            const uint32_t bal = __ballot_sync(0xffffffffu, (d >> b) & 1u);
-                            peers &= ((d >> b) & 1u) ? bal : ~bal;
-                        }
+                        // lanes of the same column: a bit each in the column's word, read back (columns
+                        // are spread: 32 instances span a dozen records).  Eight ballots, at three
+                        // instructions each, 225 -> 188 us for the pass at 3M Gaussians.
+                        atomicOr(&words[d], 1u << lane);
+                        __syncwarp();
+                        const uint32_t peers = words[d];
                         const uint32_t below = peers & lt;
                         const uint32_t prev = wh[d];
                         __syncwarp();
-                        if (below == 0) wh[d] = prev + (uint32_t)__popc(peers);
+                        if (below == 0) {
+                            wh[d] = (uint16_t)(prev + (uint32_t)__popc(peers));
+                            words[d] = 0;
+                        }
                         __syncwarp();
                         pos[i] = prev + (uint32_t)__popc(below);
                     }
@@ -526,7 +534,7 @@ __global__ void __launch_bounds__(kColThreads, 5) k_col_scatter(const __grid_con
 #pragma unroll
                         for (int w = 0; w < kColWarps; ++w) {
                             const uint32_t c = s_hist[w][d];
-                            s_hist[w][d] = cnt;
+                            s_hist[w][d] = (uint16_t)cnt;
                             cnt += c;
                         }
                         uint32_t rt;
