@@ -81,7 +81,8 @@ enum {
 /* Rasterizer constants.  gs_default_config() fills the paper's values. */
 typedef struct gs_raster_config {
     int tile_w, tile_h;       /* tile size in pixels: 16 x 16 (Sec. 6); 8 x 8 and 16 x 8 also supported */
-    int batch_depth;          /* Gaussians staged in shared memory per batch; <= tile_w * tile_h   */
+    int batch_depth;          /* in [1, tile_w * tile_h]; a hint: the render kernels stage 32
+                                 Gaussians per tile at a time whatever its value                */
     int sort_mode;            /* GS_SORT_TWO_PHASE or GS_SORT_KEY64                                */
     float alpha_min;          /* 1/255: skip blending updates with smaller alpha (App. C)          */
     float alpha_max;          /* 0.99: clamp alpha from above (App. C)                             */

@@ -105,7 +105,8 @@ def candidates(tile_shapes=TILE_SHAPES, batch_depths=BATCH_DEPTHS):
 def autotune(scenes: list, bg=(0.0, 0.0, 0.0), cands=None, steps: int = 3, sort_mode: str = "two_phase"):
     """Time the captured multi-scene step for every (tile shape, batch depth) candidate and
     return (best config, [(tile, batch_depth, ms), ...]).  Tile shapes are searched first at
-    their largest batch depth, then the batch depth at the best tile shape."""
+    their largest batch depth, then the batch depth at the best tile shape (the render kernels
+    stage 32 splats at a time whatever the depth, so the depths of one shape differ by noise)."""
     cands = cands if cands is not None else candidates()
     shapes = sorted({t for t, _ in cands}, key=lambda t: -t[0] * t[1])
     table = []
