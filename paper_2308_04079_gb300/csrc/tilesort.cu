@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const __grid_constant__ Mult
 // spread over all threads and warps: 1k Gaussians (2,000 records) 46 -> 14 us, 60k (131k records)
 // 52 -> 21, 200k at 1080p (651k records) 61 -> 32, with the count pass at 9.7 -> 16 there (a longer
 // look-back chain); from 3.7M records on the chunks are the full 2,048 as before.
-// 5 blocks per SM (51 registers, 44.7 KB of shared memory each): config 3 binning 0.865 ->
+// 5 blocks per SM (48 registers, 44.9 KB of shared memory each): config 3 binning 0.865 ->
 // 0.854 ms against 4 blocks at 64 registers.
 template <int MAXF>
 __global__ void __launch_bounds__(kColThreads, 5) k_col_scatter(const __grid_constant__ Multi<ColArgs, MAXF> m) {
