@@ -115,7 +115,8 @@ struct DepthSmallShared {
     uint32_t hist[kSmallWarps][256];
     uint16_t val[kDepthSmallMax];
     uint32_t scan[33];
-    uint32_t same, visible;
+    uint32_t same[kDepthPasses];   // per pass: its byte is the same in every key
+    uint32_t visible;
 };
 
 template <int MAXF>
@@ -130,6 +131,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_depth_small(const __grid_cons
         for (unsigned long long k = tid; p && k < a.clear.words[r]; k += kSmallThreads) p[k] = 0u;
     }
     if (tid == 0) sh.visible = 0;
+    if (tid < kDepthPasses) sh.same[tid] = 0;
     const int n = a.n;
     // a warp's keys are contiguous: item i of lane l is key w0 + 32 i + l
     const int items = (n + kSmallThreads - 1) / kSmallThreads;
@@ -147,9 +149,9 @@ __global__ void __launch_bounds__(kSmallThreads) k_depth_small(const __grid_cons
     vis = __reduce_add_sync(0xffffffffu, vis);
     __syncthreads();
     if (lane == 0 && vis) atomicAdd(&sh.visible, vis);
-    for (int shift = 0; shift < 32; shift += 8) {
+    for (int pass = 0; pass < kDepthPasses; ++pass) {
+        const int shift = 8 * pass;
         for (int k = tid; k < kSmallWarps * 256; k += kSmallThreads) (&sh.hist[0][0])[k] = 0;
-        if (tid == 0) sh.same = 0;
         __syncthreads();
         uint32_t* const wh = sh.hist[warp];
         uint32_t pos[kSmallItems];
@@ -181,11 +183,13 @@ __global__ void __launch_bounds__(kSmallThreads) k_depth_small(const __grid_cons
                 c[w] = sh.hist[w][tid];
                 cnt += c[w];
             }
-            if (cnt == (uint32_t)n) sh.same = 1;
+            if (cnt == (uint32_t)n) sh.same[pass] = 1;
         }
         uint32_t total;
         uint32_t start = block_exclusive_scan<uint32_t>(cnt, sh.scan, &total);
-        if (sh.same) continue;   // block-uniform: this byte orders nothing
+        // block-uniform: this byte orders nothing.  A flag per pass, set before the scan's barriers and
+        // never written again: a warp may read it after others have gone on to the next pass.
+        if (sh.same[pass]) continue;
         if (tid < 256) {
 #pragma unroll
             for (int w = 0; w < kSmallWarps; ++w) {
