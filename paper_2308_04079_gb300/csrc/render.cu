@@ -72,8 +72,9 @@ constexpr float kUnscale = 1.1774100225154747f;
 constexpr float kLn2 = 0.69314718055994531f;
 // Side of a sub-block in pixels: the unit of culling, contribution bits and lane groups.
 constexpr int kSub = 8;
-// Magnitude of dL/dC, colour or conic from which pixels' products are kept apart (backward_unit).
-constexpr float kWild = 1.0e30f;
+// Magnitude of dL/dC, colour or conic from which pixels' products are kept apart (backward_unit):
+// three products of two smaller values, their sum, and a conic entry times a pixel offset are finite.
+constexpr float kWild = 1.0e18f;
 
 struct Staged {
     float4 a;   // (ox, oy, thr, lo): tile-relative offset, skip threshold, log2(opacity)
@@ -653,7 +654,9 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
                 es[u] = s_e[ln.slot][k];
             }
             // care: alpha may be clamped (its gradient then stops), or a product of a pixel that
-            // does not blend the splat may not be finite (`odd` dL/dC): clear those products
+            // does not blend the splat may not be finite (`odd` dL/dC, a wild colour or conic): its
+            // terms are then cleared before they meet a sum or the pixel's recurrence, 0 x inf
+            // included.  Without care they are finite (kWild), and 0 as alpha is
             auto blend = [&](auto care_c) {
             constexpr bool care = decltype(care_c)::value;
 #pragma unroll
@@ -674,13 +677,13 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
                     float sv[2], xv[2], na[2], om[2];
                     unpack2(s, sv[0], sv[1]);
                     unpack2(x, xv[0], xv[1]);
-                    bool grad[2], grad_a[2];
+                    bool blends[2], grad[2], grad_a[2];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const float oG = hw_exp2(xv[h]);
                         const bool ok = pos < mylast[2 * i + h] && !(sv[h] > thr);
                         if (ok) ++nblend;
-                        grad[h] = ok;
+                        blends[h] = grad[h] = ok;
                         if (LIMIT) {
                             grad[h] = ok && seen[2 * i + h] >= skip[2 * i + h];
                             seen[2 * i + h] += ok;
@@ -699,13 +702,15 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
                     const f32x2 Ti = mul2(T[i], pack2(hw_rcp(om[0]), hw_rcp(om[1])));   // T_i = T_{i+1} / (1 - alpha_i)
                     f32x2 nw = mul2(na2, Ti);
                     // dL/dalpha = T_i (c_i - R_{i+1}) . dL/dC;  R_i . dL/dC = R_{i+1} . dL/dC + alpha (c_i - R_{i+1}) . dL/dC
-                    const f32x2 diff = fma2(e.r, dLr[i], fma2(e.g, dLg[i], fma2(e.b, dLb[i], nRd[i])));
+                    f32x2 diff = fma2(e.r, dLr[i], fma2(e.g, dLg[i], fma2(e.b, dLb[i], nRd[i])));
+                    if (care) diff = only(diff, blends);
                     nRd[i] = fma2(na2, diff, nRd[i]);
                     T[i] = Ti;
                     // -dL/d(power) = -alpha dL/dalpha; its sums with 1, p, p^2 (q is the row's)
-                    f32x2 ndp = mul2(nw, diff);
+                    f32x2 ndp = mul2(nw, diff), pg = p;
                     if (care) {
                         ndp = only(ndp, grad_a);
+                        pg = only(p, grad_a);
                         Gr = add2(Gr, only(mul2(nw, dLr[i]), grad));
                         Gg = add2(Gg, only(mul2(nw, dLg[i]), grad));
                         Gb = add2(Gb, only(mul2(nw, dLb[i]), grad));
@@ -718,14 +723,14 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
                         Gg = fma2(nw, dLg[i], Gg);
                         Gb = fma2(nw, dLb[i], Gb);
                     }
-                    const f32x2 ndpp = mul2(ndp, p);
+                    const f32x2 ndpp = mul2(ndp, pg);
                     S0 = add2(S0, ndp);
                     S1 = add2(S1, ndpp);
-                    S2 = fma2(ndpp, p, S2);
+                    S2 = fma2(ndpp, pg, S2);
                 }
             sums[u][0] = S0; sums[u][1] = S1; sums[u][2] = S2;
             sums[u][3] = Gr; sums[u][4] = Gg; sums[u][5] = Gb;
-            qs[u] = low(row.q);
+            qs[u] = care && (S0 | S1) == 0 ? 0.f : low(row.q);   // no term of this row: q may be infinite
             any_grad |= contrib;
             }
             };
