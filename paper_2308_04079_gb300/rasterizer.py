@@ -216,8 +216,9 @@ class Frame:
     def _binned_then(self, g: GaussianTensors, then) -> None:
         """ensure_binned with ``then()`` (launches that follow the binning on the stream) queued
         before the host waits for the binning's status, so that the GPU has work while the host
-        reads it and prepares the next call.  After a capacity overflow the binning leaves every
-        tile empty: what ``then`` launched is harmless, and it is launched again after the redo."""
+        reads it and prepares the next call.  A binning that failed leaves every tile empty: what
+        ``then`` launched is harmless, is waited for before the workspace is given up, and is
+        launched again after a redo."""
         code, st = self._bin(g, then)
         if code == abi.GS_ERR_CAPACITY:
             self._alloc(int(st.num_instances * 1.25) + 1024)
@@ -240,7 +241,12 @@ class Frame:
         then()
         read.synchronize()
         st = abi.gs_device_status.from_buffer_copy(ctypes.string_at(host.data_ptr(), nbytes))
-        return abi.status_code(st), st
+        code = abi.status_code(st)
+        if code not in (abi.GS_OK, abi.GS_ERR_NUMERIC):
+            # the caller gives the workspace up (it grows, or the error leaves it to whoever holds the
+            # frame), and the allocator knows nothing of this stream's launches on it
+            torch.cuda.current_stream().synchronize()
+        return code, st
 
 
 def _gradients_struct(grads: dict) -> abi.gs_gradients:
