@@ -60,10 +60,13 @@ def _stream() -> int:
     return torch.cuda.current_stream().cuda_stream
 
 
-def _prep(t: torch.Tensor | None, align: int = 4) -> torch.Tensor | None:
+def _prep(t: torch.Tensor | None, align: int = 4, keep: bool = True) -> torch.Tensor | None:
+    """``t`` as the kernels take it.  ``keep``: for longer than the call, so as a tensor object of its
+    own, which does not follow the caller's ``.data``, ``set_`` or ``requires_grad_`` (2 us each of
+    the 130 us of a small render, which therefore goes without)."""
     if t is None:
         return None
-    if t.requires_grad:
+    if keep or t.requires_grad:
         t = t.detach()
     if t.dtype != torch.float32:
         raise TypeError("rasterizer inputs must be float32")
@@ -89,8 +92,7 @@ class GaussianTensors:
         return int(self.means.shape[0])
 
     def prepared(self) -> "GaussianTensors":
-        return GaussianTensors(_prep(self.means), _prep(self.scales), _prep(self.quats, 16), _prep(self.opacities),
-                               _prep(self.sh), int(self.sh_degree))
+        return _prepared(self, keep=True)
 
     def struct(self) -> abi.gs_gaussians:
         g = abi.gs_gaussians()
@@ -105,6 +107,11 @@ class GaussianTensors:
             return torch.from_numpy(np.ascontiguousarray(np.asarray(a, dtype=np.float32))).to(device)
         quats = None if g.quats is None else t(g.quats)
         return GaussianTensors(t(g.means), t(g.scales), quats, t(g.opacities), t(g.sh), int(g.sh_degree))
+
+
+def _prepared(g, keep: bool) -> GaussianTensors:
+    return GaussianTensors(_prep(g.means, keep=keep), _prep(g.scales, keep=keep), _prep(g.quats, 16, keep),
+                           _prep(g.opacities, keep=keep), _prep(g.sh, keep=keep), int(g.sh_degree))
 
 
 class Frame:
@@ -337,7 +344,7 @@ def _frame_for(frame: Frame | None, n: int, camera, cfg, device) -> Frame:
 def render(g: GaussianTensors, camera, bg=(0.0, 0.0, 0.0), cfg=None, frame: Frame | None = None):
     """Forward render.  Returns (image [3,H,W], T_final [H,W], last [H,W] int32, frame); a
     given ``frame`` is reused (with this camera) when its size and constants fit."""
-    g = g.prepared()
+    g = _prepared(g, keep=False)
     frame = _frame_for(frame, g.n, camera, cfg, g.means.device)
     outs = frame.outputs()
     frame._binned_then(g, lambda: frame.render_forward(bg, *outs))

@@ -59,3 +59,35 @@ def test_a_binning_that_succeeds_is_not_waited_for_beyond_its_status(monkeypatch
     s = _Status(monkeypatch, [0])
     s.run()
     assert s.log == ["bin", "blend", "status"]
+
+
+class _Device(torch.Tensor):
+    """A host tensor that passes for a device tensor where only its attributes are looked at."""
+    is_cuda = True
+
+
+def _tensors(n=3):
+    def t(*shape):
+        return torch.rand(*shape).as_subclass(_Device)
+    return rasterizer.GaussianTensors(t(n, 3), t(n, 3), t(n, 4), t(n), t(n, 4, 3), 1)
+
+
+FIELDS = ("means", "scales", "quats", "opacities", "sh")
+
+
+def test_prepared_tensors_are_not_the_callers_own():
+    """prepared() is kept across calls (a batch's Gaussians, a forward pass's inputs until its backward
+    pass): it shares the caller's values, but not what becomes of the caller's tensor objects."""
+    g = _tensors()
+    p = g.prepared()
+    want = {k: (getattr(p, k).data_ptr(), getattr(p, k).shape) for k in FIELDS}
+    for k in FIELDS:
+        t = getattr(g, k)
+        assert t.data_ptr() == want[k][0]
+        t[0] = 2.0                                       # a new value is seen
+        assert torch.all(getattr(p, k)[0] == 2.0)
+        old = t.detach()
+        t.data = torch.zeros(1).as_subclass(_Device)     # another tensor in its place is not
+        assert (getattr(p, k).data_ptr(), getattr(p, k).shape) == want[k] == (old.data_ptr(), old.shape)
+        getattr(p, k).requires_grad_()
+        assert not t.requires_grad
