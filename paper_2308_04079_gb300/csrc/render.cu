@@ -163,9 +163,7 @@ struct Lanes {
 };
 
 // A staged splat in shared memory: what the packed arithmetic broadcasts is stored twice, so that a
-// 16-byte load yields register pairs (20 move instructions fewer per splat and warp).  Bit 31 of
-// `id` marks a splat whose pairs need care: its alpha can reach alpha_max, its conic is not finite
-// (a degenerate splat without dilation) or its colour could overflow a product.
+// 16-byte load yields register pairs (20 move instructions fewer per splat and warp).
 struct __align__(16) Entry {
     f32x2 ox, oy;         // offset of the tile's first pixel centre from the mean
     f32x2 l11, l21;       // scaled Cholesky factor of the conic
@@ -173,10 +171,10 @@ struct __align__(16) Entry {
     f32x2 r, g;           // colour
     f32x2 b;
     float ko;             // 1 / opacity
-    uint32_t id;          // Gaussian | care << 31
+    uint32_t id;          // Gaussian
 };
 
-__device__ __forceinline__ Entry entry_of(const Staged& st, float4 col, uint32_t gid, float lo_care) {
+__device__ __forceinline__ Entry entry_of(const Staged& st, float4 col, uint32_t gid) {
     Entry e;
     e.ox = pack2(st.a.x, st.a.x);
     e.oy = pack2(st.a.y, st.a.y);
@@ -188,10 +186,24 @@ __device__ __forceinline__ Entry entry_of(const Staged& st, float4 col, uint32_t
     e.g = pack2(col.y, col.y);
     e.b = pack2(col.z, col.z);
     e.ko = st.b.w;
-    const bool care = !(st.a.w <= lo_care) || !(fabsf(st.b.x) + fabsf(st.b.y) + fabsf(st.b.z) < kWild) ||
-                      !(col.x + col.y + col.z < kWild);   // colours are clamped at 0
-    e.id = gid | (care ? 0x80000000u : 0u);
+    e.id = gid;
     return e;
+}
+
+// Whether a splat's pairs need care: its alpha can reach alpha_max, its conic is not finite (a
+// degenerate splat without dilation) or its colour could overflow a product.
+__device__ __forceinline__ bool needs_care(const Staged& st, float4 col, float lo_care) {
+    return !(st.a.w <= lo_care) || !(fabsf(st.b.x) + fabsf(st.b.y) + fabsf(st.b.z) < kWild) ||
+           !(col.x + col.y + col.z < kWild);   // colours are clamped at 0
+}
+
+// A ballot of the lanes that stage a window, round r, as bits of the window's 32 positions (of the
+// lane's own tile).
+template <typename LN>
+__device__ __forceinline__ uint32_t window_bits(const LN& ln, bool v, int r) {
+    const uint32_t bal = __ballot_sync(0xffffffffu, v);
+    if (LN::SL == 32) return bal;
+    return ((bal >> (ln.slot * LN::SL & 31)) & ((1u << (LN::SL & 31)) - 1u)) << (r * LN::SL & 31);
 }
 
 // What a lane fetches of a splat it stages.
@@ -386,17 +398,19 @@ __device__ __forceinline__ void forward_unit(const RenderFwdArgs& a, uint32_t un
         const bool active = (who & gmask) != 0;                // this group
         // stage the next 32 splats of the tile; bit k of a group's word: splat base + k can
         // reach its sub-block
-        uint32_t word = 0;
+        uint32_t word = 0, careful = 0;
         __syncwarp();
 #pragma unroll
         for (int r = 0; r < LN::ROUNDS; ++r) {
             const int k = ln.tl + r * LN::SL;
             uint32_t reach = 0;
+            bool care = false;
             if (base + (uint32_t)k < len) {
                 if (!LN::AHEAD) fetch_splat(fetched, ids[r], a);
                 Staged st;
                 stage_splat(fetched.xy, fetched.conic, x0, y0, log2_amin, st);
-                s_e[ln.slot][k] = entry_of(st, fetched.rgb, fetched.id, lo_care);
+                s_e[ln.slot][k] = entry_of(st, fetched.rgb, fetched.id);
+                care = needs_care(st, fetched.rgb, lo_care);
                 const int s0 = ln.sub0();
 #pragma unroll
                 for (int s = 0; s < LN::NS; ++s) {
@@ -406,12 +420,15 @@ __device__ __forceinline__ void forward_unit(const RenderFwdArgs& a, uint32_t un
             }
 #pragma unroll
             for (int s = 0; s < LN::NS; ++s) {
-                uint32_t bal = __ballot_sync(full, (reach >> s) & 1u);
-                if (LN::SL < 32) bal = ((bal >> (ln.slot * LN::SL & 31)) & ((1u << (LN::SL & 31)) - 1u)) << (r * LN::SL & 31);
-                if (ln.group % LN::NS == s) word |= bal;
+                const uint32_t bits = window_bits(ln, (reach >> s) & 1u, r);
+                if (ln.group % LN::NS == s) word |= bits;
             }
+            if (!LN::ONE_PATH) careful |= window_bits(ln, care, r);
         }
         if (!active) word = 0;
+        // one path for the warp and the window: groups on different ones would take turns (1M opaque
+        // splats at 1080p: 176 us, so 134)
+        const bool care = LN::ONE_PATH || __any_sync(full, (word & careful) != 0);
         // in flight while this window is blended
         if (LN::AHEAD) fetch_splat(fetched, ids[0], a);
         fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, base + (LN::AHEAD ? 64u : 32u) + (uint32_t)ln.tl, len);
@@ -465,10 +482,7 @@ __device__ __forceinline__ void forward_unit(const RenderFwdArgs& a, uint32_t un
                     if (any) mb |= bit[u];
                 }
             };
-            uint32_t flags = e[0].id;
-#pragma unroll
-            for (int u = 1; u < U; ++u) flags |= e[u].id;
-            if (LN::ONE_PATH || (int)flags < 0) blend(std::true_type{});
+            if (LN::ONE_PATH || care) blend(std::true_type{});
             else blend(std::false_type{});
         }
 #pragma unroll
@@ -628,14 +642,22 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
         const uint32_t base = 32u * (uint32_t)w;
         uint32_t word = next;
         next = word_of(w - 1);
+        uint32_t careful = 0;
         __syncwarp();
 #pragma unroll
         for (int r = 0; r < LN::ROUNDS; ++r) {
             if (!LN::AHEAD) fetch_splat(fetched, ids[r], a);
             Staged st;
             stage_splat(fetched.xy, fetched.conic, x0, y0, log2_amin, st);
-            s_e[ln.slot][ln.tl + r * LN::SL] = entry_of(st, fetched.rgb, fetched.id, lo_care);
+            s_e[ln.slot][ln.tl + r * LN::SL] = entry_of(st, fetched.rgb, fetched.id);
+            if (!LN::ONE_PATH) careful |= window_bits(ln, needs_care(st, fetched.rgb, lo_care), r);
         }
+        // care: alpha may be clamped (its gradient then stops), or a product of a pixel that does not
+        // blend a splat may not be finite (`odd` dL/dC, a wild colour or conic): its terms are then
+        // cleared before they meet a sum or the pixel's recurrence, 0 x inf included.  Without care
+        // they are finite (kWild), and 0 as alpha is.  One path for the warp and the window: groups
+        // on different ones would take turns (1M opaque splats at 1080p: 267 us, so 214).
+        const bool care_w = LN::ONE_PATH || __any_sync(full, odd || (word & careful) != 0);
         // in flight while this window is walked
         if (LN::AHEAD) fetch_splat(fetched, ids[0], a);
         fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, 32u * (uint32_t)max(0, w - (LN::AHEAD ? 2 : 1)) + (uint32_t)ln.tl, len);
@@ -653,10 +675,6 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
                 word &= ~(1u << k);
                 es[u] = s_e[ln.slot][k];
             }
-            // care: alpha may be clamped (its gradient then stops), or a product of a pixel that
-            // does not blend the splat may not be finite (`odd` dL/dC, a wild colour or conic): its
-            // terms are then cleared before they meet a sum or the pixel's recurrence, 0 x inf
-            // included.  Without care they are finite (kWild), and 0 as alpha is
             auto blend = [&](auto care_c) {
             constexpr bool care = decltype(care_c)::value;
 #pragma unroll
@@ -734,10 +752,7 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
             any_grad |= contrib;
             }
             };
-            uint32_t flags = odd ? 0x80000000u : 0u;
-#pragma unroll
-            for (int u = 0; u < U; ++u) flags |= es[u].id;
-            if (LN::ONE_PATH || (int)flags < 0) blend(std::true_type{});
+            if (LN::ONE_PATH || care_w) blend(std::true_type{});
             else blend(std::false_type{});
             if (LIMIT && !__any_sync(full, any_grad)) continue;
             float v[U][9];
@@ -752,7 +767,7 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 if (at[u] != 0xffffffffu) {
-                    float* dst = grad2d + 12 * (size_t)(es[u].id & 0x7fffffffu) + slot0;
+                    float* dst = grad2d + 12 * (size_t)es[u].id + slot0;
                     if (nslots > 0) atomicAdd(dst, f0 * v[u][0]);
                     if (nslots > 1) atomicAdd(dst + 1, f1 * v[u][1]);
                 }
