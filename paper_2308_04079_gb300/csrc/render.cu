@@ -330,6 +330,9 @@ __device__ __forceinline__ f32x2 blend_pair(f32x2 s, float thr, f32x2 al, f32x2 
     return w;
 }
 
+__device__ __forceinline__ uint32_t bits_of(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ uint32_t bits_of(uint32_t v) { return v; }
+
 // Forward pass of the groups of one warp (`unit`) of a frame with ntiles tiles.
 template <int PX, int SUBS, bool COUNT>
 __device__ __forceinline__ void forward_unit(const RenderFwdArgs& a, uint32_t unit, uint32_t ntiles) {
@@ -490,26 +493,51 @@ __device__ __forceinline__ void forward_unit(const RenderFwdArgs& a, uint32_t un
         // every word the group walks is written: the backward pass reads no other
         if (active && ln.lane % LN::GL == 0) bits[(size_t)(base >> 5) * SUBS] = mb;
     }
-    const size_t P = (size_t)c.W * c.H;
+    // Out through shared memory, two planes at a time, so that consecutive lanes store consecutive
+    // pixels: stored from the lane that blended it, each pixel of a warp's store lies in a row of its
+    // own (1,000 splats at 1080p: 46 us, so 16 at any width; 3M 408 -> 406).
+    float t[PX], r[PX], g[PX], b[PX];
+#pragma unroll
+    for (int i = 0; i < LN::PAIRS; ++i) {
+        unpack2(T[i], t[2 * i], t[2 * i + 1]);
+        unpack2(Cr[i], r[2 * i], r[2 * i + 1]);
+        unpack2(Cg[i], g[2 * i], g[2 * i + 1]);
+        unpack2(Cb[i], b[2 * i], b[2 * i + 1]);
+    }
 #pragma unroll
     for (int i = 0; i < PX; ++i) {
-        const int px = px0 + i;
-        if (live && px < c.W && py < c.H) {
-            const size_t p = (size_t)py * c.W + px;
-            float r[2], g[2], b[2], tt[2];
-            unpack2(T[i / 2], tt[0], tt[1]);
-            unpack2(Cr[i / 2], r[0], r[1]);
-            unpack2(Cg[i / 2], g[0], g[1]);
-            unpack2(Cb[i / 2], b[0], b[1]);
-            const float t = fabsf(tt[i & 1]);
-            a.out_rgb[p] = r[i & 1] + t * a.bg[0];
-            a.out_rgb[P + p] = g[i & 1] + t * a.bg[1];
-            a.out_rgb[2 * P + p] = b[i & 1] + t * a.bg[2];
-            a.out_T[p] = t;
-            a.out_last[p] = last[i];
-            if (COUNT) a.out_count[p] = nblended[i];
-        }
+        t[i] = fabsf(t[i]);
+        r[i] += t[i] * a.bg[0];
+        g[i] += t[i] * a.bg[1];
+        b[i] += t[i] * a.bg[2];
     }
+    constexpr int ROW = kSub + 1, BLOCK = kSub * ROW;   // words of a row and of a sub-block (no bank conflicts)
+    static_assert(sizeof(s_e) >= 2 * LN::GW * BLOCK * sizeof(uint32_t), "two planes of the warp's sub-blocks");
+    uint32_t* const s_px = reinterpret_cast<uint32_t*>(s_e) + ln.group * (2 * BLOCK);
+    const size_t P = (size_t)c.W * c.H;
+    auto store = [&](auto* p0, const auto (&v0)[PX], auto* p1, const auto (&v1)[PX], bool second) {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < PX; ++i) {
+            uint32_t* const w = s_px + ln.row * ROW + ln.col + i;
+            w[0] = bits_of(v0[i]);
+            if (second) w[BLOCK] = bits_of(v1[i]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < PX; ++j) {
+            const int q = j * LN::GL + ln.lane % LN::GL, row = q / kSub, col = q % kSub;
+            const int x = x0 + kSub * ln.sx + col, y = y0 + kSub * ln.sy + row;
+            if (live && x < c.W && y < c.H) {
+                const size_t p = (size_t)y * c.W + x;
+                reinterpret_cast<uint32_t*>(p0)[p] = s_px[row * ROW + col];
+                if (second) reinterpret_cast<uint32_t*>(p1)[p] = s_px[BLOCK + row * ROW + col];
+            }
+        }
+    };
+    store(a.out_rgb, r, a.out_rgb + P, g, true);
+    store(a.out_rgb + 2 * P, b, a.out_T, t, true);
+    store(a.out_last, last, a.out_count, nblended, COUNT);
 }
 
 // One warp per block.  A single frame reads its arguments straight from the parameter bank; a
