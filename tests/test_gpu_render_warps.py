@@ -75,3 +75,41 @@ def test_widths_and_alignments_change_nothing(width, grad_limit):
         for k, w in wgrads.items():
             # the same terms summed in another order: fp32 sums of up to ~1e4 terms of both signs
             assert np.linalg.norm(grads[k] - w) <= 1e-5 * max(np.linalg.norm(w), 1e-30), (companion, shift, k)
+
+
+# ---- groups that walk the same splats add as one ----
+
+@pytest.mark.parametrize("tile", TILES)
+@pytest.mark.parametrize("W,H", SIZES)
+def test_splats_that_cover_every_sub_block(W, H, tile):
+    """Forty splats larger than the frame: every group of every warp walks the same positions, over a
+    full window of 32 and a partial one."""
+    from paper_2308_04079_gb300 import make_config
+    g, cam = S.tiny_scene(42, n=40, width=W, height=H, deg=1, log_scale_mean=0.7, log_scale_std=0.2)
+    g.opacities = (np.asarray(g.opacities) * 0.2).astype(np.float32)
+    _check(g, cam, (0.1, 0.3, 0.2), S.upstream_grad(43, H, W), cfg=make_config(tile=tile), ocfg=_ocfg(tile),
+           label=f"frame-filling {W}x{H} {tile[0]}x{tile[1]}")
+
+
+@pytest.mark.parametrize("tile", TILES)
+@pytest.mark.parametrize("W,H", SIZES)
+def test_tiles_with_a_splat_each(W, H, tile):
+    """One splat in the middle of every tile, within the tile: the groups of a warp that holds several
+    tiles walk the same positions of their lists, which name different splats."""
+    from paper_2308_04079_gb300 import make_config
+    tw, th = tile
+    TX, TY = W // tw, H // th
+    x, y = (v.reshape(-1) for v in np.meshgrid((np.arange(TX) + 0.5) * tw, (np.arange(TY) + 0.5) * th))
+    n = x.size
+    rng = np.random.default_rng(44)
+    z = rng.uniform(1.0, 3.0, n)
+    f = float(W)
+    quats = rng.normal(size=(n, 4))
+    g = S.Gaussians(means=np.stack([(x - W / 2) / f * z, (y - H / 2) / f * z, z], 1).astype(np.float32),
+                    scales=(rng.uniform(0.1, 0.7, (n, 3)) * z[:, None] / f).astype(np.float32),
+                    quats=(quats / np.linalg.norm(quats, axis=1, keepdims=True)).astype(np.float32),
+                    opacities=rng.uniform(0.1, 0.95, n).astype(np.float32),
+                    sh=rng.normal(0.5, 0.2, (n, 1, 3)).astype(np.float32), sh_degree=0)
+    cam = S.Camera(W, H, f, f, W / 2, H / 2, np.eye(3, dtype=np.float32), np.zeros(3, np.float32))
+    _check(g, cam, (0.0, 0.0, 0.0), S.upstream_grad(45, H, W), cfg=make_config(tile=tile), ocfg=_ocfg(tile),
+           label=f"a splat per tile {W}x{H} {tw}x{th}")
