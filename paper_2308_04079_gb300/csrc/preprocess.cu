@@ -14,8 +14,6 @@
 //   -> dL/dM = (J W)^T dL/dV -> (s, R) -> q_hat -> q (normalisation Jacobian);
 //   dL/d(J W) -> dL/dJ -> dL/dt; dL/dmean2D -> dL/dt; dL/dt -> dL/dmu = W^T dL/dt;
 //   dL/drgb (clamp mask) -> dL/dSH = Y dL/drgb and -> dL/d dir -> dL/dmu.
-#include <algorithm>
-
 #include "gs_device.cuh"
 #include "gs_kernels.h"
 
@@ -383,7 +381,17 @@ __device__ __forceinline__ void bwd_view(const PreprocessBwdArgs& a, const BwdIn
 // scene): the gradients of all the group's views are summed in registers and written once
 // (or added to the output when accumulating).  Group g owns blocks [block_base[g],
 // block_base[g+1]) and frames [frame_begin[g], frame_begin[g+1]).
+// Whether SH rows of `row` floats that are not whole 16-byte vectors are staged in shared memory.
+// A single view that overwrites its gradients, us with a row per thread -> staged, 1M Gaussians: rows
+// of 15 floats 86 -> 70, 27 152 -> 106, 45 245 -> 129.  Short rows waste little of their sectors (3
+// floats 37 -> 45, 9 47 -> 56) and the lanes of a row of a multiple of 4 meet in the banks (12 57 ->
+// 101, 48 284 -> 482).  Accumulating reads and writes every row, where a row per thread leaves alone
+// what no view saw (27 floats, every Gaussian visible: 165 -> 177, one in eight: 86 -> 172), and in a
+// batch the rows are moved once for all views (8 views of 1M, 27 floats: the pass 1655 -> 1692).
 constexpr int kStageFloats = 48;   // longest row staged: 256 rows fill 48 KB
+__host__ __device__ constexpr bool stage_rows(int row, bool accumulate) {
+    return !accumulate && row > 12 && row % 4 != 0 && row <= kStageFloats;
+}
 
 template <int DEG, bool VEC, int MAXF, bool ISO>
 __global__ void __launch_bounds__(256) k_preprocess_backward_t(const __grid_constant__ BwdPlan<MAXF> m) {
@@ -403,11 +411,11 @@ __global__ void __launch_bounds__(256) k_preprocess_backward_t(const __grid_cons
     const int first = (int)(blockIdx.x - m.block_base[g]) * blockDim.x;   // the block's first Gaussian
     const int i = first + threadIdx.x;
     const int row = a.sh_stride * 3;   // floats per Gaussian in the SH buffers
-    // Rows that are not whole 16-byte vectors (degrees 0 and 2) go through shared memory: the block's
-    // rows are one contiguous run, moved with consecutive lanes on consecutive words, where a row
-    // per thread left every 32-byte sector to eight instructions (500k Gaussians of degree 2: 76 us).
+    // Staged rows (degree 2, stage_rows): the block's rows are one contiguous run, moved with
+    // consecutive lanes on consecutive words, where a row per thread left every 32-byte sector to
+    // eight instructions (500k Gaussians of degree 2: 76 -> 40 us).
     extern __shared__ __align__(16) float s_rows[];
-    const bool staged = !VEC && row <= kStageFloats;
+    const bool staged = !VEC && MAXF == 1 && stage_rows(row, a.accumulate != 0);
     const int run = min((int)blockDim.x, a.n - first) * row;
     if (staged) {
         const float* src = a.sh + (size_t)first * row;
@@ -472,16 +480,9 @@ __global__ void __launch_bounds__(256) k_preprocess_backward_t(const __grid_cons
         __syncthreads();
         float* dst = a.g_sh + (size_t)first * row;
         const int quads = (reinterpret_cast<uintptr_t>(dst) & 15) == 0 ? run / 4 : 0;
-        for (int k = threadIdx.x; k < quads; k += blockDim.x) {
-            float4 v = reinterpret_cast<const float4*>(s_rows)[k];
-            float4* d = reinterpret_cast<float4*>(dst) + k;
-            if (a.accumulate) {
-                const float4 o = *d;
-                v = make_float4(o.x + v.x, o.y + v.y, o.z + v.z, o.w + v.w);
-            }
-            *d = v;
-        }
-        for (int k = 4 * quads + threadIdx.x; k < run; k += blockDim.x) dst[k] = a.accumulate ? dst[k] + s_rows[k] : s_rows[k];
+        for (int k = threadIdx.x; k < quads; k += blockDim.x)
+            reinterpret_cast<float4*>(dst)[k] = reinterpret_cast<const float4*>(s_rows)[k];
+        for (int k = 4 * quads + threadIdx.x; k < run; k += blockDim.x) dst[k] = s_rows[k];
         if (i >= a.n) return;
     }
     if (!any && a.accumulate) return;   // no view saw it: nothing to add
@@ -586,10 +587,6 @@ void preprocess_deg(const PrePlan<MAXF>& m, bool vec, cudaStream_t s) {
 
 template <typename M>
 cudaError_t launch_rows(void (*kernel)(M), dim3 grid, size_t smem, const M& m, cudaStream_t s) {
-    if (smem > 32 * 1024) {   // with the static argument copy of a batch it may pass 48 KB
-        const cudaError_t e = cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
     kernel<<<grid, 256, smem, s>>>(m);
     return cudaGetLastError();
 }
@@ -597,14 +594,11 @@ cudaError_t launch_rows(void (*kernel)(M), dim3 grid, size_t smem, const M& m, c
 template <int DEG, int MAXF>
 cudaError_t preprocess_bwd_deg(const BwdPlan<MAXF>& m, bool vec, cudaStream_t s) {
     const dim3 grid(m.block_base[m.groups]);
-    // shared memory for the groups whose rows are staged (with a batch's arguments beside it)
-    size_t smem = 0;
-    if (!vec)
-        for (int g = 0; g < m.groups; ++g) {
-            const int row = 3 * m.a[m.frame_begin[g]].sh_stride;
-            if (row <= kStageFloats) smem = std::max(smem, (size_t)256 * row * sizeof(float));
-        }
-    if (m.a[0].cfg.isotropic) {
+    const PreprocessBwdArgs& a = m.a[0];
+    // shared memory for staged rows (at most 256 x 48 floats, the 48 KB of any launch)
+    const int row = 3 * a.sh_stride;
+    const size_t smem = !vec && MAXF == 1 && stage_rows(row, a.accumulate != 0) ? (size_t)256 * row * sizeof(float) : 0;
+    if (a.cfg.isotropic) {
         if (vec) return launch_rows(k_preprocess_backward_t<DEG, true, MAXF, true>, grid, smem, m, s);
         return launch_rows(k_preprocess_backward_t<DEG, false, MAXF, true>, grid, smem, m, s);
     }
