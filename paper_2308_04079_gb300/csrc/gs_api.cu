@@ -280,20 +280,32 @@ gs_status preprocess_impl(const FrameSet<MAXF>& fs, const gs_gaussians* g, cudaS
     gs_status st = clear_regions(fs, clr, s);
     if (st != GS_OK) return st;
     // one launch per (SH degree, SH row alignment) class of frames; frames that render the same
-    // Gaussians with the same kernel form a group
+    // Gaussians with the same kernel form a group, where that fills the chip
     bool done[MAXF] = {};
     for (int v0 = 0; v0 < fs.count; ++v0) {
         if (done[v0]) continue;
         PrePlan<MAXF> m;
         m.groups = 0;
         int nf = 0;
+        auto same_class = [&](int u) {
+            return g[u].sh_degree == g[v0].sh_degree &&
+                   sh_vec(g[u].sh, g[u].sh_stride) == sh_vec(g[v0].sh, g[v0].sh_stride);
+        };
+        bool share = false;
+        if (MAXF > 1) {
+            long long blocks = 0;   // of the class, each scene once
+            for (int u = v0; u < fs.count; ++u) {
+                bool first = same_class(u);
+                for (int v = v0; v < u && first; ++v) first = !same_gaussians(g[u], g[v]);
+                if (first) blocks += (g[u].n + 255) / 256;
+            }
+            share = preprocess_shares_views(blocks);
+        }
         for (int u = v0; u < fs.count; ++u) {
-            if (done[u] || g[u].sh_degree != g[v0].sh_degree ||
-                sh_vec(g[u].sh, g[u].sh_stride) != sh_vec(g[v0].sh, g[v0].sh_stride))
-                continue;
+            if (done[u] || !same_class(u)) continue;
             m.frame_begin[m.groups++] = nf;
             for (int v = u; v < fs.count; ++v) {
-                if (done[v] || !same_gaussians(g[u], g[v])) continue;
+                if (done[v] || (v != u && !(share && same_gaussians(g[u], g[v])))) continue;
                 done[v] = true;
                 const gs_frame* f = fs.f[v];
                 const Layout& L = fs.L[v];

@@ -378,6 +378,8 @@ int persistent_blocks(int threads) {
     return blocks;
 }
 template <int MAXF> cudaError_t launch_preprocess(PrePlan<MAXF>& m, cudaStream_t s);
+// Whether the views of a scene form one group, in a launch of `blocks` blocks if they do.
+bool preprocess_shares_views(long long blocks);
 template <int MAXF> cudaError_t launch_preprocess_backward(BwdPlan<MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_depth_small(const Multi<DepthSmallArgs, MAXF>& m, cudaStream_t s);
 template <int MAXF> cudaError_t launch_depth_hist(Multi<DepthHistArgs, MAXF>& m, cudaStream_t s);

@@ -14,6 +14,8 @@
 //   -> dL/dM = (J W)^T dL/dV -> (s, R) -> q_hat -> q (normalisation Jacobian);
 //   dL/d(J W) -> dL/dJ -> dL/dt; dL/dmean2D -> dL/dt; dL/dt -> dL/dmu = W^T dL/dt;
 //   dL/drgb (clamp mask) -> dL/dSH = Y dL/drgb and -> dL/d dir -> dL/dmu.
+#include <type_traits>
+
 #include "gs_device.cuh"
 #include "gs_kernels.h"
 
@@ -142,26 +144,27 @@ __device__ __forceinline__ void ld_v8(const float* p, float (&v)[8]) {
 // 6 blocks of 256 per SM (40 registers): config 3 (3M Gaussians) 0.157 -> 0.148 ms against the
 // 48-register build at 5 blocks; streaming or L2-only loads of the SH rows were slower (0.194,
 // 0.175 ms) and also slowed the backward, which re-reads the rows that stay in L2.
-// A batch's views of one scene go through one thread per Gaussian: its parameters and its SH row
-// come from L1 after the first view (as 16 sets of blocks, 16 views of 1M Gaussians read the 236 MB
-// of parameters 16 times: 796 -> 635 us; 4 scenes of 3 views 201 -> 176).  What bounds it then is
-// the instructions of the projection at half the warps (64 registers), not HBM.
-template <int DEG, bool VEC, int MAXF, bool ISO>
-__global__ void __launch_bounds__(256, MAXF == 1 ? 6 : 4) k_preprocess_t(const __grid_constant__ PrePlan<MAXF> m) {
+// VIEWS: a batch's views of one scene go through one thread per Gaussian: its parameters and its SH
+// row come from L1 after the first view (as 16 sets of blocks, 16 views of 1M Gaussians read the 236
+// MB of parameters 16 times: 796 -> 635 us; 4 scenes of 3 views 201 -> 176).  What bounds it then is
+// the instructions of the projection at half the warps (64 registers), not HBM; so a scene that
+// leaves SMs without blocks is worked through view by view (preprocess_shares_views).
+template <int DEG, bool VEC, int MAXF, bool ISO, bool VIEWS>
+__global__ void __launch_bounds__(256, VIEWS ? 4 : 6) k_preprocess_t(const __grid_constant__ PrePlan<MAXF> m) {
     constexpr int D = (DEG + 1) * (DEG + 1);
     const int g = find_frame<MAXF>(m.block_base, m.groups, blockIdx.x);
     const int f0 = m.frame_begin[g], f1 = m.frame_begin[g + 1];
     // a batch reads its group's arguments from a shared copy (generic loads otherwise)
-    __shared__ __align__(16) PreprocessArgs s_args[MAXF > 1 ? MAXF : 1];
+    __shared__ __align__(16) PreprocessArgs s_args[VIEWS ? MAXF : 1];
     if (MAXF > 1) {
-        const int words = (int)(sizeof(PreprocessArgs) / 4) * (f1 - f0);
+        const int words = (int)(sizeof(PreprocessArgs) / 4) * (VIEWS ? f1 - f0 : 1);
         for (int k = threadIdx.x; k < words; k += blockDim.x)
             reinterpret_cast<uint32_t*>(s_args)[k] = reinterpret_cast<const uint32_t*>(&m.a[f0])[k];
         __syncthreads();
     }
     const PreprocessArgs& a0 = MAXF == 1 ? m.a[0] : s_args[0];   // Gaussians shared by the group
     const int i = (int)(blockIdx.x - m.block_base[g]) * blockDim.x + threadIdx.x;
-    const int n = a0.n, nv = MAXF == 1 ? 1 : f1 - f0;   // a single frame: straight-line code
+    const int n = a0.n, nv = VIEWS ? f1 - f0 : 1;   // a view per group: straight-line code
     for (int v = 0; v < nv; ++v) {
         const PreprocessArgs& a = MAXF == 1 ? m.a[0] : s_args[v];
         bool visible = false;
@@ -573,15 +576,15 @@ bool sh_vectorisable(const float* sh, int sh_stride, const float* gsh = nullptr)
     return base && (3 * sh_stride) % 4 == 0;
 }
 
-template <int DEG, int MAXF>
+template <int DEG, int MAXF, bool VIEWS>
 void preprocess_deg(const PrePlan<MAXF>& m, bool vec, cudaStream_t s) {
     const dim3 grid(m.block_base[m.groups]);
     if (m.a[0].cfg.isotropic) {
-        if (vec) k_preprocess_t<DEG, true, MAXF, true><<<grid, 256, 0, s>>>(m);
-        else k_preprocess_t<DEG, false, MAXF, true><<<grid, 256, 0, s>>>(m);
+        if (vec) k_preprocess_t<DEG, true, MAXF, true, VIEWS><<<grid, 256, 0, s>>>(m);
+        else k_preprocess_t<DEG, false, MAXF, true, VIEWS><<<grid, 256, 0, s>>>(m);
     } else {
-        if (vec) k_preprocess_t<DEG, true, MAXF, false><<<grid, 256, 0, s>>>(m);
-        else k_preprocess_t<DEG, false, MAXF, false><<<grid, 256, 0, s>>>(m);
+        if (vec) k_preprocess_t<DEG, true, MAXF, false, VIEWS><<<grid, 256, 0, s>>>(m);
+        else k_preprocess_t<DEG, false, MAXF, false, VIEWS><<<grid, 256, 0, s>>>(m);
     }
 }
 
@@ -612,18 +615,42 @@ cudaError_t preprocess_bwd_deg(const BwdPlan<MAXF>& m, bool vec, cudaStream_t s)
 template <int MAXF>
 cudaError_t launch_preprocess(PrePlan<MAXF>& m, cudaStream_t s) {
     m.block_base[0] = 0;
-    for (int g = 0; g < m.groups; ++g)
+    bool views = false;   // some group has several
+    for (int g = 0; g < m.groups; ++g) {
         m.block_base[g + 1] = m.block_base[g] + (uint32_t)((m.a[m.frame_begin[g]].n + 255) / 256);
+        views |= m.frame_begin[g + 1] - m.frame_begin[g] > 1;
+    }
     if (m.block_base[m.groups] == 0) return cudaSuccess;
     const PreprocessArgs& a = m.a[0];
     const bool vec = sh_vectorisable(a.sh, a.sh_stride);
-    switch (a.sh_degree) {
-        case 0: preprocess_deg<0>(m, vec, s); break;
-        case 1: preprocess_deg<1>(m, vec, s); break;
-        case 2: preprocess_deg<2>(m, vec, s); break;
-        default: preprocess_deg<3>(m, vec, s); break;
+    auto launch = [&](auto views_c) {
+        constexpr bool V = decltype(views_c)::value;
+        switch (a.sh_degree) {
+            case 0: preprocess_deg<0, MAXF, V>(m, vec, s); break;
+            case 1: preprocess_deg<1, MAXF, V>(m, vec, s); break;
+            case 2: preprocess_deg<2, MAXF, V>(m, vec, s); break;
+            default: preprocess_deg<3, MAXF, V>(m, vec, s); break;
+        }
+    };
+    if constexpr (MAXF > 1) {
+        if (views) launch(std::true_type{});
+        else launch(std::false_type{});
+    } else {
+        launch(std::false_type{});
     }
     return cudaGetLastError();
+}
+
+// A block that works through all views holds its SM for as many blocks' time, so what counts is how
+// full the waves of resident blocks (608 on 152 SMs) are: 0.9 of them, 0.8 of three, any more.  Views on
+// their own -> together, 16 views of degree 3, us: 60k Gaussians (0.39 waves) 57 -> 68, 130k (0.84)
+// 106 -> 123, 145k (0.93) 121 -> 124 (degree 0 71 -> 70), 160k (1.03) 127 -> 150, 200k (1.29) 157 ->
+// 205, 260k (1.67) 206 -> 221, 300k (1.93) 265 -> 236, 320k (2.06) 259 -> 264, 420k (2.7) 354 -> 319,
+// 1M (6.4, its parameters larger than L2) 880 -> 716.
+bool preprocess_shares_views(long long blocks) {
+    const long long wave = persistent_blocks<k_preprocess_t<3, true, kMaxFrames, false, true>>(256);
+    const long long waves = (blocks + wave - 1) / wave;
+    return waves > 3 || 10 * blocks >= (waves < 3 ? 9 : 8) * waves * wave;
 }
 
 template <int MAXF>
