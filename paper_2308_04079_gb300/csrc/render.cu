@@ -430,8 +430,9 @@ __device__ __forceinline__ void forward_unit(const RenderFwdArgs& a, uint32_t un
         }
         if (!active) word = 0;
         // one path for the warp and the window: groups on different ones would take turns (1M opaque
-        // splats at 1080p: 176 us, so 134)
-        const bool care = LN::ONE_PATH || __any_sync(full, (word & careful) != 0);
+        // splats at 1080p: 176 us, so 134); a group's own choice per iteration where blended splats are
+        // counted, as care costs more there (3M: 459 us the one way, 450 the other)
+        const bool care = LN::ONE_PATH || (!COUNT && __any_sync(full, (word & careful) != 0));
         // in flight while this window is blended
         if (LN::AHEAD) fetch_splat(fetched, ids[0], a);
         fetch_ids<LN::ROUNDS, LN::SL>(ids, vals, base + (LN::AHEAD ? 64u : 32u) + (uint32_t)ln.tl, len);
@@ -485,7 +486,11 @@ __device__ __forceinline__ void forward_unit(const RenderFwdArgs& a, uint32_t un
                     if (any) mb |= bit[u];
                 }
             };
-            if (LN::ONE_PATH || care) blend(std::true_type{});
+            uint32_t mine = 0;
+            if (COUNT && !LN::ONE_PATH)
+#pragma unroll
+                for (int u = 0; u < U; ++u) mine |= bit[u] & careful;
+            if (LN::ONE_PATH || care || mine) blend(std::true_type{});
             else blend(std::false_type{});
         }
 #pragma unroll
@@ -556,14 +561,15 @@ __global__ void __launch_bounds__(32, 16) k_render_forward_t(const __grid_consta
 }
 
 // A lane's PX consecutive pixels of one plane (src: the first), 0 outside the image (`in` pixels are
-// inside).  Quads or pairs where the alignment allows (W a multiple, the caller's buffer): eight loads
-// of one pixel each read a sector eight times, from L2 where the rows' stride makes them share a cache
-// set (1,000 splats at 1080p: 33 us, so 24).
+// inside), as quads or pairs if `wide`: eight loads of one pixel each read a sector eight times, from L2
+// where the rows' stride makes them share a cache set (1,000 splats at 1080p: 33 us, so 24).
+template <int PX>
+constexpr int kRowVec = PX >= 4 ? 4 : 2;
 template <int PX, typename T>
-__device__ __forceinline__ void load_row(const T* src, int in, T (&v)[PX]) {
-    constexpr int VEC = PX >= 4 ? 4 : 2;
+__device__ __forceinline__ void load_row(const T* src, int in, bool wide, T (&v)[PX]) {
+    constexpr int VEC = kRowVec<PX>;
     struct __align__(sizeof(T) * VEC) Vec { T e[VEC]; };
-    if (in == PX && reinterpret_cast<uintptr_t>(src) % sizeof(Vec) == 0) {
+    if (wide) {
 #pragma unroll
         for (int i = 0; i < PX; i += VEC) {
             const Vec x = *reinterpret_cast<const Vec*>(src + i);
@@ -622,12 +628,23 @@ __device__ __forceinline__ void backward_unit(const RenderBwdArgs& a, uint32_t u
     const int in = live && py < c.H ? min(PX, max(0, c.W - px0)) : 0;   // the lane's pixels inside the image
     const size_t first = in ? (size_t)py * c.W + px0 : 0;
     float tf[PX], dr_[PX], dg_[PX], db_[PX];
-    load_row<PX>(a.last + first, in, mylast);
-    load_row<PX>(a.T_final + first, in, tf);
-    load_row<PX>(a.dL_drgb + first, in, dr_);
-    load_row<PX>(a.dL_drgb + P + first, in, dg_);
-    load_row<PX>(a.dL_drgb + 2 * P + first, in, db_);
-    if (LIMIT) load_row<PX>(a.count + first, in, skip);
+    auto wide = [&](const void* p) { return in == PX && reinterpret_cast<uintptr_t>(p) % (4 * kRowVec<PX>) == 0; };
+    auto load = [&](auto wide_of) {
+        load_row<PX>(a.last + first, in, wide_of(a.last + first), mylast);
+        load_row<PX>(a.T_final + first, in, wide_of(a.T_final + first), tf);
+        load_row<PX>(a.dL_drgb + first, in, wide_of(a.dL_drgb + first), dr_);
+        load_row<PX>(a.dL_drgb + P + first, in, wide_of(a.dL_drgb + P + first), dg_);
+        load_row<PX>(a.dL_drgb + 2 * P + first, in, wide_of(a.dL_drgb + 2 * P + first), db_);
+    };
+    if constexpr (LIMIT) {   // short of registers: one choice for all planes (500k Limited-BW 179 -> 177 us)
+        if (wide(a.last + first) && wide(a.T_final + first) && wide(a.dL_drgb + first) && wide(a.dL_drgb + P + first))
+            load([](const void*) { return true; });
+        else
+            load([](const void*) { return false; });
+        load_row<PX>(a.count + first, in, false, skip);
+    } else {
+        load(wide);
+    }
 #pragma unroll
     for (int i = 0; i < PX; ++i) {
         mylast[i] = min(mylast[i], len);   // last positions never exceed the tile's list
