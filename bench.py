@@ -53,7 +53,7 @@ KERNEL_NAMES = {"preprocess": "k_preprocess_t", "render_forward": "k_render_forw
 # DRAM bytes (ncu dram__bytes_read.sum + dram__bytes_write.sum) of one launch of each
 # single-kernel stage on the 3M-Gaussian 1080p frame, taken from a capture of the current
 # kernel; a stage without such a capture reports None.
-TRAFFIC = {"render_backward_tiles": 107_399_680, "render_forward": 57_036_288}
+TRAFFIC = {"render_backward_tiles": 107_509_248, "render_forward": 60_736_000}
 
 
 def env_int(k, d):

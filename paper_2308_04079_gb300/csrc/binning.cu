@@ -15,12 +15,12 @@
 //   bits, Gaussian index) order, exactly the order the 64-bit sort produces.
 //
 // Radix sort: one kernel per digit pass in the onesweep style (Merrill & Grimshaw's radix
-// sorting, single-pass with decoupled look-back): every block claims a 4096-key chunk from an
-// atomic counter (chunks are claimed in order, so a block only ever waits on chunks already
-// held by running blocks), ranks its keys with warp-private shared-memory digit counters,
-// publishes per-digit counts, resolves its global digit offsets by looking
-// back over predecessor chunks (bounded spin), stages the keys in shared memory in local sorted
-// order and writes them out coalesced.  Digit histograms of every pass are computed up front
+// sorting, single-pass with decoupled look-back): every block claims a chunk of 1024 to 4096 keys
+// (sort_items; 3072 of 64 bits) from an atomic counter (chunks are claimed in order, so a block only
+// ever waits on chunks already held by running blocks), ranks its keys with warp-private
+// shared-memory digit counters, publishes per-digit counts, resolves its global digit offsets by
+// looking back over predecessor chunks (bounded spin), stages the keys in shared memory in local
+// sorted order and writes them out coalesced.  Digit histograms of every pass are computed up front
 // (fused into the kernel that produces the keys).
 #include <algorithm>
 #include <type_traits>

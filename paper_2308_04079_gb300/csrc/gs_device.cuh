@@ -88,13 +88,8 @@ __device__ __forceinline__ int clampi(int x, int lo, int hi) { return x < lo ? l
 // error grows like sqrt(lambda_max / lambda_min) of Sigma' instead of lambda_max / lambda_min
 // (the expanded form cancels along the major axis of elongated splats).  With
 // Sigma' = [[A, B], [B, C]] and D = det Sigma': l11 = sqrt(C / D), l21 = -B / sqrt(C D),
-// l22 = 1 / sqrt(C).  Written with explicit round-to-nearest intrinsics so that the forward
-// and backward kernels evaluate it with the same operation sequence.
-__device__ __forceinline__ float splat_power(float dx, float dy, float4 L, float& p, float& q) {
-    p = __fmaf_rn(L.y, dy, __fmul_rn(L.x, dx));
-    q = __fmul_rn(L.z, dy);
-    return __fmul_rn(-0.5f, __fmaf_rn(p, p, __fmul_rn(q, q)));
-}
+// l22 = 1 / sqrt(C).  The forward and backward kernels evaluate it with the same operation sequence
+// in explicit round-to-nearest arithmetic (stage_splat, splat_row in render.cu).
 
 // Offset of a tile's first pixel centre from a splat mean stored as an unevaluated sum
 // m = hi + lo (the preprocess stores u and v that way): (x0 + 0.5 - hi) - lo.  The first difference is exact
@@ -240,13 +235,6 @@ __device__ __forceinline__ bool reach_row(const Reach& e, float u, float v, int 
     txa = max(x0, pa >> tw_log2);          // arithmetic shift: floor division
     txb = min(x1, (pb >> tw_log2) + 1);
     return txa < txb;
-}
-
-// alpha = min(alpha_max, o * G), G = exp(power).  Returns o * G (unclamped) in oG.
-__device__ __forceinline__ float splat_alpha(float power, float o, float alpha_max, float& G, float& oG) {
-    G = __expf(power);
-    oG = __fmul_rn(o, G);
-    return fminf(alpha_max, oG);
 }
 
 // Real spherical harmonics, bands 0..3, Condon-Shortley phase, unit direction (x, y, z),

@@ -272,7 +272,7 @@ struct DepthSmallArgs {
 //   row_key = row << 17 | length << 8 | first column
 // (row < 4096, length <= 255, column <= 254).  The records, emitted in depth order, are
 // stable-sorted by row (1 or 2 byte passes of k_onesweep over the segments, not the instances);
-// then per chunk of kSortTile row-sorted records: per-tile instance counts and, per column,
+// then per chunk of 256 to 2048 row-sorted records (col_chunk): per-tile instance counts and, per column,
 // the counts of the chunk's last row (look-back inside a row); a scan of the tile counts gives
 // the ranges; the column pass expands the records into instances and stable-ranks them by
 // column within their row, writing each to its final slot.

@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(256, VIEWS ? 4 : 6) k_preprocess_t(const __gri
             } else if (project_mean(mu, c, p) && (q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w) > 0.f) {
                 project_cov(s, q, c, a.cfg.dilation, p);
                 if (p.det > 0.f) {
-                    // Cholesky factor of the conic (see splat_power).
+                    // Cholesky factor of the conic (gs_device.cuh).
                     co = make_float4(sqrtf(p.C / p.det), -p.B / sqrtf(p.C * p.det), 1.0f / sqrtf(p.C), o);
                     const float m = 0.5f * (p.A + p.C);
                     const float h = 0.5f * (p.A - p.C);

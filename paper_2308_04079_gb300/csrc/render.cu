@@ -39,8 +39,9 @@
 //   by its minor axis and their major-axis part, which the scale along the long axis needs, is
 //   lost to cancellation in fp32 sums over many pixels; in the whitened frame every direction of
 //   the splat has the same scale.  q being the row's, a lane sums dL/dpower with 1, p and p^2 over
-//   its pixels and multiplies by q and q^2 once; the nine sums of a group's lanes are reduced by a
-//   transposed reduce-scatter and every lane adds the one or two totals it holds.
+//   its pixels and multiplies by q and q^2 once; the nine sums of a group's lanes (of all the warp's,
+//   when its groups walk the same splats) are reduced by a transposed reduce-scatter and every lane
+//   adds the one or two totals it holds.
 //
 // Limited-BW (cfg.grad_limit = N > 0, the ablation of Sec. 7.3): the forward pass also records
 // the number of blended splats of every pixel (COUNT); the backward pass (LIMIT) keeps the
@@ -923,12 +924,12 @@ cudaError_t backward_px(Multi<RenderBwdArgs, MAXF>& m, cudaStream_t s) {
 // instructions per splat (four sub-blocks share a warp's iteration) but give one warp per 16x16
 // tile: a frame of few tiles leaves the chip idle behind its longest lists.  Measured, 8 / 4 / 2
 // pixels per lane, forward and backward in us:
-//   16 tiles (64x64, 5k Gaussians, 64 sub-blocks)        162 /  97 /  63    302 / 183 / 134
-//   813x611 in 8x8 tiles (60k, 7,854)                     78 /  59 /  51
-//   979x546 (150k, 8,680)                                136 / 104 /  89    161 / 136 / 152
-//   1601x901 in 16x8 tiles (500k, 22,826)                151 / 142 / 160    178 / 188 / 205
-//   1920x1080 (200k, 32,640)                             185 / 200 / 234    275 / 311 / 410
-//   1920x1080 (3M, 32,640)                               270 / 299 / 341    419 / 470 / 606
+//   16 tiles (64x64, 5k Gaussians, 64 sub-blocks)        176 / 115 /  74    283 / 177 / 133
+//   813x611 in 8x8 tiles (60k, 7,854)                     80 /  57 /  45    109 /  90 /  87
+//   979x546 (150k, 8,680)                                125 /  90 /  84    154 / 123 / 145
+//   1601x901 in 16x8 tiles (500k, 22,826, Limited-BW)    140 / 138 / 160    177 / 173 / 211
+//   1920x1080 (200k, 32,640)                             165 / 180 / 217    239 / 285 / 376
+//   1920x1080 (3M, 32,640)                               263 / 285 / 333    406 / 470 / 593
 int forward_px_for(unsigned long long groups) { return groups < 12000 ? 2 : groups < 26000 ? 4 : 8; }
 int backward_px_for(unsigned long long groups) { return groups < 3000 ? 2 : groups < 16000 ? 4 : 8; }
 
