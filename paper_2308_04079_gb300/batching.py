@@ -1,6 +1,7 @@
 """Multi-scene batches: several scenes, each seen from several views, rendered forward and
 backward as one FrameBatch (one launch per kernel for all frames), the whole step captured in
-one CUDA graph, and an autotuner that picks the tile shape and the per-tile batch depth.
+one CUDA graph, and an autotuner that picks the tile shape (and a batch depth, which no kernel
+reads: see autotune).
 
 The rasterizer's arithmetic is the single-frame one: a batch changes how the work is launched,
 never what a frame computes.  Each scene's gradients are the sum over its views."""
